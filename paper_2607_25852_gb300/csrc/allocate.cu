@@ -1,5 +1,5 @@
 // allocate.cu -- D-cut verification-depth allocation (Section 4.2 of arxiv
-// 2607.25852) in one CTA on sm_103a.
+// 2607.25852) in one CTA, or one thread-block cluster, on sm_103a.
 //
 // At most SPEC_MAX_ALLOC_POSITIONS = 8192 positions, so the whole problem fits
 // in shared memory.  Every position (i, k) becomes one 64-bit key
@@ -12,20 +12,17 @@
 // Batches of at most 1024 requests and 1024 draft positions take
 // allocate_small_kernel (below), which sorts the draft keys alone: a merge
 // tree over the per-request runs padded to a power of two when they fit in
-// 1024 slots, else a bitonic sort.  Larger batches take allocate_kernel:
-// because s_{i,k} is non-increasing in k, each request's K+1 keys already form
-// a run sorted in descending order.  A merge tree of ceil(log2 B) levels sorts
-// the B runs: at every level each key finds its place in the merged pair by
-// one binary search in the partner run.  An inclusive scan of floor(s * 2^40)
-// in sorted order then gives every candidate's utility U(T) = prefix[T - 1]
-// exactly; the first maximiser of U / cost is chosen and the kept prefixes
-// are packed densely.
+// 1024 slots, else a bitonic sort.  Larger batches take
+// allocate_cluster_kernel: up to eight CTAs sort 1024 draft keys each and rank
+// them against one another through distributed shared memory.  Sums of
+// floor(s * 2^40) over the top positions give every candidate's utility U(T)
+// exactly; the first maximiser of U / cost is chosen and the kept prefixes are
+// packed densely.
 #include <float.h>
 #include <limits.h>
 #include <math.h>
 
 #include <algorithm>
-#include <atomic>
 
 #include "spec_internal.cuh"
 
@@ -72,50 +69,92 @@ __device__ __forceinline__ long long block_inclusive_scan(long long x, long long
   return x + before;
 }
 
-// Shared-memory layout (dynamic): two key buffers of N entries, then
-// pos_base [B] int64, the confidences [B][K] fp32 at the odd row stride K | 1
-// (so that the threads of a warp, one request each, read distinct banks), the
-// draft tokens [B*K] int32 and last_tokens [B] int32.
-struct AllocSmem {
-  unsigned long long* keys[2];
-  float* conf;
-  int32_t* drafts;
-  int32_t* last;
-  long long* pos;
+// units * 2^-40 as a double, for 0 < units < 2^53 (exact), with integer
+// operations only: the product's exponent and mantissa fields are set directly.
+__device__ __forceinline__ double units_to_double(long long units) {
+  const int msb = 63 - __clzll(units);
+  const unsigned long long mant = ((unsigned long long)units << (63 - msb)) << 1 >> 12;  // the bits below the msb
+  const unsigned long long expo = (unsigned long long)(msb - 40 + 1023);
+  return __longlong_as_double((long long)((expo << 52) | mant));
+}
+
+// ---------------------------------------------------------------------------
+// Batches of more than 1024 draft positions or 1024 requests
+// ---------------------------------------------------------------------------
+// One thread-block cluster of C = ceil(max(B * K, B) / 1024) <= 8 CTAs, one
+// draft key per thread: CTA c owns the draft slots e = i * K + (k - 1) in
+// [1024 c, 1024 c + 1024) and the requests of that index range.  A single CTA
+// is bound by its serial searches (eight keys a thread) and by shared-memory
+// bank conflicts; eight CTAs take one key a thread and exchange through
+// distributed shared memory, which one GPC's SMs reach without a trip to L2.
+//   1. scores and keys of the CTA's slots; a merge tree over the per-request
+//      runs (already descending) sorts them locally;
+//   2. every CTA copies the others' sorted keys and finds each of its keys'
+//      rank among all draft keys (C - 1 interleaved binary searches);
+//   3. U(T_m) is the sum of the CTAs' local prefixes at rank T_m - B, exact
+//      in integers in any order; every CTA gets all parts and picks the same T;
+//   4. the last kept draft of each request gives its depth, sent to every
+//      CTA; each scans all depths and packs its own slots.
+// Three cluster barriers in all.  Measured at B = 256, K = 31, M = 16, calls
+// replayed from a graph: 69.4 us a call with a one-CTA merge tree over all
+// keys, 15.2 us with the cluster.  The line to allocate_small_kernel is 1024
+// draft keys because that kernel's single CTA has one key a thread up to
+// there: its sort needs no cluster barrier and no second search (7.5 us at
+// B = 64, K = 16).
+constexpr int kClusterMax = 8;
+constexpr int kSlots = kAllocThreads;  // draft slots, and requests, per CTA
+// Floats that stage the confidences of the requests a CTA's slots touch, a row
+// of K | 1 each: at most 1024 / K + 2 rows, (1024 / K + 2)(K + 1) <= 2052.
+constexpr int kConfStage = 2080;
+
+__device__ __forceinline__ void cluster_sync_all() {
+  asm volatile("barrier.cluster.arrive.release;\n\tbarrier.cluster.wait.acquire;" ::: "memory");
+}
+// The address of `local` (a shared-memory address of this CTA) in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t cluster_addr(uint32_t local, int rank) {
+  uint32_t a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"(local), "r"(rank));
+  return a;
+}
+__device__ __forceinline__ unsigned long long ldc_u64(uint32_t addr) {
+  unsigned long long v;
+  asm volatile("ld.shared::cluster.u64 %0, [%1];" : "=l"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ int ldc_s32(uint32_t addr) {
+  int v;
+  asm volatile("ld.shared::cluster.s32 %0, [%1];" : "=r"(v) : "r"(addr));
+  return v;
+}
+__device__ __forceinline__ void stc_u64(uint32_t addr, unsigned long long v) {
+  asm volatile("st.shared::cluster.u64 [%0], %1;" ::"r"(addr), "l"(v) : "memory");
+}
+__device__ __forceinline__ void stc_s32(uint32_t addr, int v) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr), "r"(v) : "memory");
+}
+
+struct ClusterSmem {
+  unsigned long long all[kClusterMax][kSlots];  // every CTA's sorted keys
+  unsigned long long keys[2][kSlots];           // local merge tree; then the prefix sums
+  long long contrib[kClusterMax][SPEC_MAX_CANDIDATES];
+  long long warp_tot[32];
+  float conf[kConfStage];                       // [i - i0][k - 1] at (i - i0) * (K | 1) + k - 1, then the scores
+  int rank[kSlots];                             // rank of the sorted keys, ascending
+  int slot_rank[kSlots];                        // rank of slot 1024 c + t
+  int depth[SPEC_MAX_ALLOC_POSITIONS];          // n_i of every request, then the row offsets
+  int best_c;
 };
 
-__device__ __forceinline__ AllocSmem carve(unsigned char* base, int N, int BK, int B) {
-  AllocSmem s;
-  s.keys[0] = reinterpret_cast<unsigned long long*>(base);
-  s.keys[1] = s.keys[0] + N;
-  unsigned char* p = reinterpret_cast<unsigned char*>(s.keys[1] + N);
-  s.pos = reinterpret_cast<long long*>(p);
-  p += (size_t)B * 8;
-  s.conf = reinterpret_cast<float*>(p);
-  p += BK > 0 ? (size_t)(BK + B) * 4 : 0;
-  s.drafts = reinterpret_cast<int32_t*>(p);
-  p += (size_t)BK * 4;
-  s.last = reinterpret_cast<int32_t*>(p);
-  return s;
-}
-
-size_t allocate_smem_bytes(int B, int K) {
-  const size_t N = (size_t)B * (K + 1), BK = (size_t)B * K;
-  // at most 24 N + 8 B + 16 bytes <= 229,392 for N <= 8192 (K = 0 needs no
-  // confidences: 16 N + 12 B + 16)
-  return N * 16 + (size_t)B * 8 + (BK > 0 ? (BK + B) * 4 : 0) + BK * 4 + (size_t)B * 4 + 16;
-}
-
-__global__ void __launch_bounds__(kAllocThreads) allocate_kernel(const AllocLaunch p) {
+template <int C>
+__global__ void __launch_bounds__(kAllocThreads, 1) allocate_cluster_kernel(const AllocLaunch p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
-  const int B = p.B, K = p.K, N = B * (K + 1), BK = B * K, L0 = K + 1;
-  const int CS = K | 1;  // odd row stride of the staged confidences
-  const AllocSmem sm = carve(smem_raw, N, BK, B);
-  __shared__ long long warp_tot[32];
-  __shared__ int sh_best_c;
-  __shared__ int sh_bad;
-  const int tid = threadIdx.x;
-  if (tid == 0) sh_bad = 0;
+  ClusterSmem& sm = *reinterpret_cast<ClusterSmem*>(smem_raw);
+  const int B = p.B, K = p.K, NK = B * K, CS = K | 1;
+  const int tid = threadIdx.x, c = blockIdx.x;
+  const int e0 = c * kSlots;                              // first slot, and first request, of this CTA
+  const int nloc = max(0, min(kSlots, NK - e0));          // draft slots here
+  const int i0 = nloc > 0 ? e0 / K : 0;                   // requests the slots touch: i0 ..
+  const int nreq = nloc > 0 ? (e0 + nloc - 1) / K - i0 + 1 : 0;
   // The next kernel (the streaming pass) may launch now: it waits for this
   // one's completion before it reads the depths and row offsets.
   pdl_launch_dependents();
@@ -124,157 +163,229 @@ __global__ void __launch_bounds__(kAllocThreads) allocate_kernel(const AllocLaun
   // only once that kernel has completed.
   pdl_wait_prerequisites();
 
-  // ---- every global input in one round trip, coalesced ----
-  for (int q = tid; q < BK; q += kAllocThreads) {
-    const int i = q / K;
-    sm.conf[q + i * (CS - K)] = p.conf[q];  // [i][k] at i * CS + k
-    sm.drafts[q] = p.drafts[q];
-  }
-  for (int i = tid; i < B; i += kAllocThreads) {
-    sm.last[i] = p.last_tokens[i];
-    sm.pos[i] = p.pos_base[i];
-  }
+  // ---- every global input in one round trip ----
+  const int nconf = nreq > 0 ? e0 + nloc - i0 * K : 0;  // <= 1024 + K - 1
+  for (int x = tid; x < nconf; x += kAllocThreads) sm.conf[x / K * CS + x % K] = p.conf[i0 * K + x];
+  const int e = e0 + tid;                               // this thread's slot ...
+  const int si = tid < nloc ? e / K : 0;                // ... of request si,
+  const int sk = tid < nloc ? e - si * K + 1 : 0;       // draft sk
+  const int draft = tid < nloc ? p.drafts[e] : 0;
+  const long long spos = tid < nloc ? p.pos_base[si] : 0;
+  const int last = e < B ? p.last_tokens[e] : 0;        // and the request e0 + tid
+  const long long rpos = e < B ? p.pos_base[e] : 0;
+  for (int i = tid; i < B; i += kAllocThreads) sm.depth[i] = 0;
   __syncthreads();
 
-  // ---- Eq. (dcut-score): fp32 prefix products; run i holds request i ----
-  for (int i = tid; i < B; i += kAllocThreads) {
+  // ---- Eq. (dcut-score): fp32 prefix products in order, a request a thread ----
+  for (int rr = tid; rr < nreq; rr += kAllocThreads) {
+    float* row = sm.conf + rr * CS;
+    const int kend = min(K, nconf - rr * K);
     float s = 1.0f;
-    sm.keys[0][i * L0] = position_key(s, 0, i);
-    for (int k = 1; k <= K; ++k) {
-      float c = sm.conf[i * CS + (k - 1)];
-      if (!(c >= 0.0f && c <= 1.0f)) {
-        sh_bad = 1;
-        c = 0.0f;
+    bool bad = false;
+#pragma unroll 4
+    for (int k = 0; k < kend; ++k) {
+      float cf = row[k];
+      if (!(cf >= 0.0f && cf <= 1.0f)) {
+        bad = true;
+        cf = 0.0f;
       }
       // -0 passes the range check and equals 0, but its sign bit would put
       // its key above every positive score: -0 + 0 = +0 drops the sign.
-      c = __fadd_rn(c, 0.0f);
-      s = __fmul_rn(s, c);
-      sm.keys[0][i * L0 + k] = position_key(s, k, i);
+      cf = __fadd_rn(cf, 0.0f);
+      s = __fmul_rn(s, cf);
+      row[k] = s;
     }
+    if (bad) report(p.status, SPEC_ERR_BAD_INPUT);
   }
   __syncthreads();
 
-  // ---- merge tree over the B sorted runs (descending) ----
-  // Level l merges runs of L = L0 * 2^l keys; position e lies in run
-  // (e / L0) >> l.  N <= 8192, so 32-bit indices suffice.
-  // The two key buffers by their shared-window addresses, so that every
-  // probe of the searches is a shared-memory load (ld.shared).
+  // ---- local merge tree (descending).  At level l the groups of 2^l runs
+  // merge in pairs; the first and the last run may be cut by the CTA's range.
+  // A key's place is its index in its group plus the number of the partner
+  // group's keys above it (keys are unique). ----
+  unsigned long long x = tid < nloc ? position_key(sm.conf[(si - i0) * CS + sk - 1], sk, si) : 0ull;
   const uint32_t kbuf0 = (uint32_t)__cvta_generic_to_shared(sm.keys[0]);
   const uint32_t kbuf1 = (uint32_t)__cvta_generic_to_shared(sm.keys[1]);
-  int cur = 0;
-  for (int lev = 0, L = L0; L < N; ++lev, L *= 2) {
-    const uint32_t in = cur ? kbuf1 : kbuf0, out = cur ? kbuf0 : kbuf1;
-    for (int e = tid; e < N; e += kAllocThreads) {
-      const int run = (e / L0) >> lev;
-      const int start = run * L;
-      const int pstart = (run ^ 1) * L;
-      const unsigned long long x = lds_u64(in + 8u * (uint32_t)e);
-      if (pstart >= N) {  // unpaired last run: copied through
-        sts_u64(out + 8u * (uint32_t)e, x);
-        continue;
+  uint32_t src = kbuf0, dst = kbuf1;
+  sts_u64(src + 8u * (uint32_t)tid, x);  // pad slots hold key 0, below every real key
+  sts_u64(dst + 8u * (uint32_t)tid, x);
+  __syncthreads();
+  const int cut = i0 * K - e0;  // <= 0: local slot of request i0's first draft
+  for (int lev = 0; (1 << lev) < nreq; ++lev) {
+    if (tid < nloc) {
+      // the request of the key now at slot tid: groups are contiguous, so the
+      // slot's own group is found from its position
+      const int group = ((tid - cut) / K) >> lev, pg = group ^ 1;
+      const int start = max(0, cut + (group << lev) * K);
+      const int pstart = max(0, cut + (pg << lev) * K);
+      const int pend = min(nloc, cut + ((pg + 1) << lev) * K);
+      int lo = pstart, n = max(0, pend - pstart);
+      while (n > 0) {
+        const int half = n >> 1;
+        const bool above = lds_u64(src + 8u * (uint32_t)(lo + half)) > x;
+        lo = above ? lo + half + 1 : lo;
+        n = above ? n - half - 1 : half;
       }
-      const int plen = min(N, pstart + L) - pstart;
-      // number of partner keys greater than x (the partner run is descending)
-      int lo = 0, hi = plen;
-      while (lo < hi) {
-        const int mid = (lo + hi) >> 1;
-        if (lds_u64(in + 8u * (uint32_t)(pstart + mid)) > x) lo = mid + 1;
-        else hi = mid;
-      }
-      sts_u64(out + 8u * (uint32_t)(min(start, pstart) + (e - start) + lo), x);
+      sts_u64(dst + 8u * (uint32_t)(min(start, pstart) + (tid - start) + (lo - pstart)), x);
     }
     __syncthreads();
-    cur ^= 1;
+    const uint32_t t = src;
+    src = dst;
+    dst = t;
+    x = lds_u64(src + 8u * (uint32_t)tid);
   }
-  const unsigned long long* keys = sm.keys[cur];
-  long long* prefix = reinterpret_cast<long long*>(sm.keys[cur ^ 1]);  // free buffer
+  if (C > 1) {
+    sm.all[c][tid] = x;
+    cluster_sync_all();
+    // ---- the other CTAs' sorted keys, then this key's rank among them ----
+#pragma unroll
+    for (int o = 1; o < C; ++o) {
+      const int cc = (c + o) & (C - 1);
+      sm.all[cc][tid] = ldc_u64(cluster_addr((uint32_t)__cvta_generic_to_shared(&sm.all[cc][tid]), cc));
+    }
+    __syncthreads();
+  }
+  int rank = tid;
+  if (C > 1) {
+    uint32_t base[C];
+    int cnt[C];
+#pragma unroll
+    for (int o = 1; o < C; ++o) {
+      base[o] = (uint32_t)__cvta_generic_to_shared(sm.all[(c + o) & (C - 1)]);
+      cnt[o] = 0;
+    }
+#pragma unroll
+    for (int step = kSlots >> 1; step > 0; step >>= 1)
+#pragma unroll
+      for (int o = 1; o < C; ++o)
+        if (lds_u64(base[o] + 8u * (uint32_t)(cnt[o] + step - 1)) > x) cnt[o] += step;
+#pragma unroll
+    for (int o = 1; o < C; ++o) {
+      if (lds_u64(base[o] + 8u * (uint32_t)cnt[o]) > x) ++cnt[o];
+      rank += cnt[o];
+    }
+  }
+  const int xi = 0xFFFF - (int)(x & 0xFFFFull);
+  const int xk = 0xFFFF - (int)((x >> 16) & 0xFFFFull);
+  sm.rank[tid] = tid < nloc ? rank : INT_MAX;  // ascending along the local order
+  if (tid < nloc) sm.slot_rank[xi * K + (xk - 1) - e0] = rank;
 
-  // ---- inclusive scan of floor(s * 2^40) in sorted order ----
-  const int per = (N + kAllocThreads - 1) / kAllocThreads;
-  const int q0 = tid * per;
-  long long local = 0;
-  for (int q = q0; q < q0 + per && q < N; ++q)
-    local += (long long)__float2ll_rd(__uint_as_float((unsigned)(keys[q] >> 32)) * 0x1p40f);
-  const long long incl = block_inclusive_scan(local, warp_tot);
-  long long run = incl - local;
-  for (int q = q0; q < q0 + per && q < N; ++q) {
-    run += (long long)__float2ll_rd(__uint_as_float((unsigned)(keys[q] >> 32)) * 0x1p40f);
-    prefix[q] = run;
-  }
+  // ---- inclusive scan of floor(s * 2^40) in the local order; the CTA's part
+  // of every U(T_m), sent to all CTAs ----
+  const long long q40 =
+      tid < nloc ? (long long)__float2ll_rd(__uint_as_float((unsigned)(x >> 32)) * 0x1p40f) : 0;
+  const long long incl = block_inclusive_scan(q40, sm.warp_tot);
+  long long* prefix = reinterpret_cast<long long*>(sm.keys[0]);
+  prefix[tid] = incl;
   __syncthreads();
+  if (tid < p.M) {
+    const int td = p.cand_T[tid] - B;  // draft positions kept at this budget
+    int lo = 0, n = nloc;              // local keys of rank < td
+    while (n > 0) {
+      const int half = n >> 1;
+      const bool below = sm.rank[lo + half] < td;
+      lo = below ? lo + half + 1 : lo;
+      n = below ? n - half - 1 : half;
+    }
+    const long long part = lo > 0 ? prefix[lo - 1] : 0;
+    const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&sm.contrib[c][tid]);
+#pragma unroll
+    for (int o = 0; o < C; ++o) {
+      if (C > 1) stc_u64(cluster_addr(mine, o), (unsigned long long)part);
+      else sm.contrib[c][tid] = part;
+    }
+  }
+  if (C > 1) cluster_sync_all();
+  else __syncthreads();
 
-  // ---- Eq. (dcut-select): first maximiser of U / cost ----
+  // ---- Eq. (dcut-select): first maximiser of U / cost, in every CTA ----
   if (tid < 32) {
-    // one lane per candidate (M <= 64: two per lane); the first maximiser
-    // in candidate order wins ties, as a sequential scan would
-    double best_obj = -INFINITY;
+    long long best_key = -1;
     int best_c = INT_MAX;
-    for (int c = tid; c < p.M; c += 32) {
-      const double U = ldexp((double)prefix[p.cand_T[c] - 1], -40);
-      if (p.utility_out) p.utility_out[c] = U;
-      const double obj = U / p.cand_cost[c];
-      if (obj > best_obj) {  // c increases along the lane's loop
-        best_obj = obj;
-        best_c = c;
+    for (int m = tid; m < p.M; m += 32) {
+      long long Uq = (long long)B << 40;
+#pragma unroll
+      for (int o = 0; o < C; ++o) Uq += sm.contrib[o][m];
+      const double U = units_to_double(Uq);
+      if (p.utility_out && c == 0) p.utility_out[m] = U;
+      // U > 0 and cost > 0: the quotients order as their bit patterns do
+      const long long obj = __double_as_longlong(U / p.cand_cost[m]);
+      if (obj > best_key) {  // m increases along the lane's loop
+        best_key = obj;
+        best_c = m;
       }
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-      const double ob = __shfl_xor_sync(0xFFFFFFFFu, best_obj, o);
+      const long long ob = __shfl_xor_sync(0xFFFFFFFFu, best_key, o);
       const int cb = __shfl_xor_sync(0xFFFFFFFFu, best_c, o);
-      if (ob > best_obj || (ob == best_obj && cb < best_c)) {
-        best_obj = ob;
+      if (ob > best_key || (ob == best_key && cb < best_c)) {
+        best_key = ob;
         best_c = cb;
       }
     }
-    if (tid == 0) sh_best_c = best_c == INT_MAX ? 0 : best_c;
+    if (tid == 0) sm.best_c = best_c == INT_MAX ? 0 : best_c;
   }
   __syncthreads();
-  const int T = p.cand_T[sh_best_c];
+  const int T = p.cand_T[sm.best_c];
+  const int TD = T - B;
 
-  // ---- keep depths: count the selected positions per request ----
-  int* counts = reinterpret_cast<int*>(prefix);  // prefix no longer needed
-  int* offsets = counts + B;                       // [B]
-  for (int i = tid; i < B; i += kAllocThreads) counts[i] = 0;
-  __syncthreads();
-  for (int q = tid; q < T; q += kAllocThreads) atomicAdd(&counts[0xFFFF - (int)(keys[q] & 0xFFFFull)], 1);
-  __syncthreads();
-
-  // ---- row offsets: exclusive scan of (n_i + 1) = counts ----
-  const int perB = (B + kAllocThreads - 1) / kAllocThreads;
-  const int b0 = tid * perB;
-  long long lsum = 0;
-  for (int i = b0; i < b0 + perB && i < B; ++i) lsum += counts[i];
-  const long long bincl = block_inclusive_scan(lsum, warp_tot);
-  long long off = bincl - lsum;
-  for (int i = b0; i < b0 + perB && i < B; ++i) {
-    offsets[i] = (int)off;
-    p.row_offsets_out[i] = (int)off;
-    p.depth_out[i] = counts[i] - 1;
-    off += counts[i];
+  // ---- keep depths: the last kept draft of each request, to every CTA ----
+  const bool kept = tid < nloc && sm.slot_rank[tid] < TD;
+  if (kept) {
+    bool next = false;
+    if (sk < K) {  // slot e + 1, in the next CTA past this one's last slot
+      if (tid + 1 < kSlots) next = sm.slot_rank[tid + 1] < TD;
+      else if (C > 1) next = ldc_s32(cluster_addr((uint32_t)__cvta_generic_to_shared(&sm.slot_rank[0]), c + 1)) < TD;
+    }
+    if (!next) {
+      const uint32_t d = (uint32_t)__cvta_generic_to_shared(&sm.depth[si]);
+#pragma unroll
+      for (int o = 0; o < C; ++o) {
+        if (C > 1) stc_s32(cluster_addr(d, o), sk);
+        else sm.depth[si] = sk;
+      }
+    }
   }
-  if (tid == kAllocThreads - 1) {
-    p.row_offsets_out[B] = (int)bincl;
+  if (C > 1) cluster_sync_all();
+  else __syncthreads();
+
+  // ---- row offsets: exclusive scan of (n_i + 1) over all requests, in every
+  // CTA; each writes its requests' outputs ----
+  const int per = (B + kAllocThreads - 1) / kAllocThreads;  // <= 8, consecutive requests a thread
+  const int b0 = min(B, tid * per), b1 = min(B, b0 + per);
+  int sum = 0;
+  for (int i = b0; i < b1; ++i) sum += sm.depth[i] + 1;
+  int off = (int)block_inclusive_scan(sum, sm.warp_tot) - sum;
+  for (int i = b0; i < b1; ++i) {
+    const int n = sm.depth[i];
+    if (i / kSlots == c) {
+      p.row_offsets_out[i] = off;
+      p.depth_out[i] = n;
+    }
+    sm.depth[i] = off;  // the offsets from here on
+    off += n + 1;
+  }
+  if (c == 0 && tid == 0) {
+    p.row_offsets_out[B] = T;  // sum of (n_i + 1): the T kept positions
     *p.chosen_T_out = T;
   }
   __syncthreads();
 
   // ---- dense packing of the kept prefixes ----
-  for (int q = tid; q < N; q += kAllocThreads) {
-    if (q < T) {
-      const unsigned long long key = keys[q];
-      const int i = 0xFFFF - (int)(key & 0xFFFFull);
-      const int k = 0xFFFF - (int)((key >> 16) & 0xFFFFull);
-      const int row = offsets[i] + k;
-      p.packed_tokens_out[row] = k == 0 ? sm.last[i] : sm.drafts[i * K + (k - 1)];
-      p.packed_pos_out[row] = sm.pos[i] + k;
-    } else {
-      p.packed_tokens_out[q] = -1;
-      p.packed_pos_out[q] = -1;
-    }
+  if (e < B) {
+    p.packed_tokens_out[sm.depth[e]] = last;
+    p.packed_pos_out[sm.depth[e]] = rpos;
   }
-  if (tid == 0 && sh_bad) report(p.status, SPEC_ERR_BAD_INPUT);
+  if (kept) {
+    const int row = sm.depth[si] + sk;
+    p.packed_tokens_out[row] = draft;
+    p.packed_pos_out[row] = spos + sk;
+  }
+  for (int r = T + e; r < B * (K + 1); r += C * kAllocThreads) {
+    p.packed_tokens_out[r] = -1;
+    p.packed_pos_out[r] = -1;
+  }
 }
 
 // ---------------------------------------------------------------------------
@@ -291,15 +402,6 @@ __global__ void __launch_bounds__(kAllocThreads) allocate_kernel(const AllocLaun
 // ranks without atomics: draft (i, k) in the top T - B, with (i, k + 1) not,
 // ends request i's kept prefix.
 constexpr int kSmallSlots = kAllocThreads;
-
-// units * 2^-40 as a double, for 0 < units < 2^53 (exact), with integer
-// operations only: the product's exponent and mantissa fields are set directly.
-__device__ __forceinline__ double units_to_double(long long units) {
-  const int msb = 63 - __clzll(units);
-  const unsigned long long mant = ((unsigned long long)units << (63 - msb)) << 1 >> 12;  // the bits below the msb
-  const unsigned long long expo = (unsigned long long)(msb - 40 + 1023);
-  return __longlong_as_double((long long)((expo << 52) | mant));
-}
 
 __device__ __forceinline__ unsigned long long shfl_xor_u64(unsigned long long x, int o) {
   const unsigned lo = __shfl_xor_sync(0xFFFFFFFFu, (unsigned)x, o);
@@ -550,31 +652,40 @@ __global__ void __launch_bounds__(kAllocThreads) allocate_small_kernel(const All
 
 bool allocate_is_small(int B, int K) { return B <= kSmallSlots && (long long)B * K <= kSmallSlots; }
 
+// One cluster of C CTAs (B and B * K are at most 1024 C), launched behind the
+// previous kernel as launch_after_previous does.
+template <int C>
+static cudaError_t launch_cluster(const AllocLaunch& p, cudaStream_t stream) {
+  cudaError_t err = cudaFuncSetAttribute(allocate_cluster_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                         (int)sizeof(ClusterSmem));
+  if (err != cudaSuccess) return err;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3(C);
+  cfg.blockDim = dim3(kAllocThreads);
+  cfg.dynamicSmemBytes = sizeof(ClusterSmem);
+  cfg.stream = stream;
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributeClusterDimension;
+  attr[1].val.clusterDim = {C, 1, 1};
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  err = cudaLaunchKernelEx(&cfg, allocate_cluster_kernel<C>, p);
+  return err != cudaSuccess ? err : cudaGetLastError();
+}
+
 cudaError_t launch_allocate(const AllocLaunch& p, cudaStream_t stream) {
   cudaError_t err;
   if (allocate_is_small(p.B, p.K)) {
     err = launch_after_previous(allocate_small_kernel, dim3(1), dim3(kAllocThreads), 0, stream, p);
     return err != cudaSuccess ? err : cudaGetLastError();
   }
-  // The dynamic shared memory limit is raised once per device, to the
-  // largest size asked for so far.
-  const size_t smem = allocate_smem_bytes(p.B, p.K);
-  constexpr int kMaxDevices = 64;
-  static std::atomic<size_t> raised[kMaxDevices];
-  int dev = -1;
-  err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  if (dev < 0 || dev >= kMaxDevices || raised[dev].load(std::memory_order_relaxed) < smem) {
-    err = cudaFuncSetAttribute(allocate_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (err != cudaSuccess) return err;
-    if (dev >= 0 && dev < kMaxDevices) {
-      size_t cur = raised[dev].load(std::memory_order_relaxed);
-      while (cur < smem && !raised[dev].compare_exchange_weak(cur, smem)) {
-      }
-    }
-  }
-  err = launch_after_previous(allocate_kernel, dim3(1), dim3(kAllocThreads), smem, stream, p);
-  return err != cudaSuccess ? err : cudaGetLastError();
+  const int slots = std::max(p.B * p.K, p.B);
+  if (slots <= kSlots) return launch_cluster<1>(p, stream);
+  if (slots <= 2 * kSlots) return launch_cluster<2>(p, stream);
+  if (slots <= 4 * kSlots) return launch_cluster<4>(p, stream);
+  return launch_cluster<8>(p, stream);
 }
 
 }  // namespace spec

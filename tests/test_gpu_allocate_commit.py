@@ -91,6 +91,28 @@ def test_random_allocations(B, K):
         assert_alloc_equal(g, r)
 
 
+# The cluster kernel: one, two, four and eight CTAs, requests cut at a CTA's
+# 1024 slots (K not dividing 1024, up to K = 255), CTAs without draft slots
+# ((1025, 0), (8192, 0)), one slot past a CTA ((205, 5), (1025, 1)), a full
+# last CTA ((512, 15)) and up to eight requests a thread in the offset scan.
+@pytest.mark.parametrize("B,K", [(1025, 0), (1025, 1), (4096, 1), (2730, 2), (342, 3), (205, 5), (1100, 6), (256, 15),
+                                 (60, 18), (256, 31), (63, 129), (40, 200), (5, 255), (32, 255)])
+def test_cluster_allocations(B, K):
+    rng = np.random.default_rng(B * 31 + K)
+    N = B * (K + 1)
+    for conf in (rng.choice([0.0, 0.5, 1.0], size=(B, K)), rng.beta(6.0, 1.0, size=(B, K)), np.ones((B, K))):
+        conf = conf.astype(np.float32)
+        Ts = [int(x) for x in rng.integers(B, N + 1, size=10)] + [N, B]  # in no order, some equal
+        costs = list(rng.uniform(0.5, 3.0, len(Ts)))
+        last = torch.as_tensor(rng.integers(0, 10**6, B), dtype=torch.int32)
+        drafts = torch.as_tensor(rng.integers(0, 10**6, (B, K)), dtype=torch.int32)
+        pos = torch.as_tensor(rng.integers(0, 10**9, B), dtype=torch.int64)
+        g = gpu_allocate(torch.as_tensor(conf), Ts, costs, last, drafts, pos)
+        r = oracle.allocate(conf, Ts, costs, last.numpy(), drafts.numpy(), pos.numpy())
+        assert_alloc_equal(g, r)
+        assert int(g["status"][0]) == 0
+
+
 @pytest.mark.parametrize("B,K", [(4, 3), (64, 16), (300, 7)])
 def test_negative_zero_confidences(B, K):
     """-0 confidences (the value 0, sign bit set) rank as zero scores: the
