@@ -11,19 +11,22 @@
 //   c_{k+1} = q_k(z_{k+1}) at tau'
 //   s_0 = 1, s_k = fl32(s_{k-1} * c_k)
 //
-// draft_rows_kernel: one CTA per (row, chunk of equal size).  Each
-// warp takes a round of 8 consecutive race blocks (256 entries each; 4 for
-// fp32) at a time: lane l loads entries 8l..8l+7 of each, the round's max
-// comes from one redux over order-preserving integer keys, and the blocks'
-// sums of 2^(l*c2 - fl(M_r*c2)) from one transposed butterfly, after which
-// each group of lanes owns one block.  Level 1 of the race compares blocks in
-// the log2 domain,
+// draft_rows_kernel: one warp per (row, segment of race blocks), warps
+// independent of one another.  A warp takes a round of 8 consecutive race
+// blocks (256 entries each; 4 for fp32) at a time: a group of 8 lanes reads
+// whole 128-byte lines of one block, so a block's sum of
+// 2^(l*c2 - fl(M_r*c2)) needs three shuffles inside its lane group; the
+// round's max M_r comes from one redux over order-preserving integer keys.
+// Level 1 of the race compares blocks in the log2 domain,
 //   log2 key_b = log2 E_b - log2 sum_b - M_r*c2   (see BlockKey),
-// so no pass over the row is needed before the draw.  The row's softmax
-// statistics merge from the rounds' (M_r, sum_r).  The last CTA of a row to
-// arrive merges the chunks, draws the entry inside the winning block (level
-// 2) and writes z, c and the row statistics; the last row of a request to
-// finish writes the scores.
+// so no pass over the row is needed before the draw.  Each lane keeps the sum
+// of one block of every 32, forms that block's key once, and holds its own
+// best block and its own part of the softmax sum until the segment ends: no
+// other exchange sits between a round's loads and the next.  The last warp of
+// a row to arrive merges the segments, draws the entry inside the winning
+// block (level 2; at tau = 0 finds the first maximum inside the round that
+// holds it) and writes z, c and the row statistics; the last row of a request
+// to finish writes the scores.
 #include <float.h>
 #include <math.h>
 
@@ -33,8 +36,11 @@
 
 namespace spec {
 
-constexpr int kDraftThreads = 256;
+constexpr int kDraftThreads = 128;
+constexpr int kDraftCtas = 8;       // resident CTAs per SM (32 warps, 64 registers a thread)
+constexpr int kDraftSlots = 152 * kDraftCtas * kDraftThreads / 32;  // warps in one wave
 constexpr int kSegmentBlocks = 64;  // race blocks per warp unit, at most
+constexpr int kGroup = 32;          // race blocks whose level-1 words one warp-wide Philox call gives
 
 // A level-1 candidate: block idx with L = log2 E_b - log2 sum_b and block
 // max M, i.e. log2 key = L - M*c2.  Two candidates compare by
@@ -55,7 +61,7 @@ struct alignas(16) DraftPartial {
   float m;        // max logit of the chunk
   float s;        // sum of 2^(l*c2 - fl(m*c2))
   float key;      // tau > 0: L of the best block; tau = 0: the max (= m)
-  int32_t idx;    // tau > 0: the best block; tau = 0: lowest argmax (INT_MAX: none)
+  int32_t idx;    // tau > 0: the best block; tau = 0: first block of the first round that holds the max (INT_MAX: none)
   int32_t flags;  // bit0: NaN or +inf seen
   float keyM;     // tau > 0: M of the best block
   int32_t pad[2];
@@ -90,11 +96,14 @@ static inline long long ceil_div_ll(long long a, long long b) { return (a + b - 
 static DraftGeometry draft_geometry(int B, int K, int V) {
   DraftGeometry g{};
   const long long R = (long long)B * K;
-  // one warp per (row, segment): segments of about 64 blocks (8 rounds),
-  // split evenly in steps of 8 blocks
+  // one warp per (row, segment): segments of a whole number of 8 blocks, as
+  // many as fill one wave of warps (B = 16, K = 16, V = 128256: 17.5 us; twice
+  // and four times as many 18.2 and 20.6 us), or of at most kSegmentBlocks when
+  // the rows fill several (32 or 64 blocks: the same time at the stress size)
   const long long nb = ceil_div_ll(V, 256);
-  const long long ns = std::max(1LL, ceil_div_ll(nb, kSegmentBlocks));
-  const long long bps = std::min<long long>(kSegmentBlocks, ceil_div_ll(ceil_div_ll(nb, ns), 8) * 8);
+  const long long want = std::max(8LL, std::min<long long>(kSegmentBlocks, ceil_div_ll(ceil_div_ll(R * nb, kDraftSlots), 8) * 8));
+  const long long ns = ceil_div_ll(nb, want);
+  const long long bps = ceil_div_ll(ceil_div_ll(nb, ns), 8) * 8;
   g.NC = (int)ceil_div_ll(nb, bps);
   g.chunk = (int)(bps * 256);
   g.part_off = 0;
@@ -116,239 +125,208 @@ __device__ __forceinline__ int orderable(float f) {
 }
 __device__ __forceinline__ float from_orderable(int k) { return __int_as_float(k < 0 ? k ^ 0x7FFFFFFF : k); }
 
-// A lane's 8 entries 8l..8l+7 of a race block as raw 16-byte words (one for
-// bf16, two for fp32), and their unpacking; entries at or past V read -inf.
+// A round's 16-byte words: lane l reads, for each of the round's kHalf sets of
+// four blocks, word l & 7 of every 128-byte line of block 4h + (l >> 3): 8
+// loads in flight, each of four whole lines over the warp.
 template <typename T>
-struct Lane8;
+struct Round;
 template <>
-struct Lane8<__nv_bfloat16> {
-  static constexpr int kWords = 1;
-  static constexpr int kBlocksPerRound = 8;  // two Philox quads
-  template <bool kVec>
-  __device__ static void load(const __nv_bfloat16* row, int v8, int V, uint4 (&w)[kWords]) {
-    if (kVec) {
-      w[0] = v8 < V ? ldg_stream(row + v8) : make_uint4(0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u, 0xFF80FF80u);
-    } else {
-      uint32_t h[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        h[e] = v8 + e < V ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(row) + v8 + e) : 0xFF80u;
-      w[0] = make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
-    }
-  }
-  __device__ static void unpack(const uint4 (&w)[kWords], float (&x)[8]) {
-    x[0] = bf16_lo(w[0].x), x[1] = bf16_hi(w[0].x), x[2] = bf16_lo(w[0].y), x[3] = bf16_hi(w[0].y);
-    x[4] = bf16_lo(w[0].z), x[5] = bf16_hi(w[0].z), x[6] = bf16_lo(w[0].w), x[7] = bf16_hi(w[0].w);
-  }
-  // max over the lane's entries of N blocks as a tree of packed bf16 maxima
-  // (a NaN loses to any number here; the sums catch it)
-  template <int N>
-  __device__ static float round_max(const uint4 (&w)[N][kWords]) {
-    __nv_bfloat162 m[N];
-#pragma unroll
-    for (int u = 0; u < N; ++u) {
-      const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&w[u][0]);
-      m[u] = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
-    }
-#pragma unroll
-    for (int n = N / 2; n > 0; n >>= 1)
-#pragma unroll
-      for (int u = 0; u < n; ++u) m[u] = __hmax2(m[u], m[u + n]);
-    return fmaxf(__low2float(m[0]), __high2float(m[0]));
-  }
+struct Round<__nv_bfloat16> {
+  static constexpr int kBlocks = 8;  // race blocks per round
+  static constexpr int kHalf = 2;    // sets of four
+  static constexpr int kLines = 4;   // 128-byte lines per block
+  static constexpr int kPer = 8;     // entries per word
+  static constexpr uint32_t kPad = 0xFF80FF80u;
 };
 template <>
-struct Lane8<float> {
-  static constexpr int kWords = 2;
-  static constexpr int kBlocksPerRound = 4;  // one Philox quad
-  template <bool kVec>
-  __device__ static void load(const float* row, int v8, int V, uint4 (&w)[kWords]) {
-    const uint32_t ninf = 0xFF800000u;
-    if (kVec) {
-      w[0] = v8 < V ? ldg_stream(row + v8) : make_uint4(ninf, ninf, ninf, ninf);
-      w[1] = v8 < V ? ldg_stream(row + v8 + 4) : make_uint4(ninf, ninf, ninf, ninf);
-    } else {
-      uint32_t h[8];
-#pragma unroll
-      for (int e = 0; e < 8; ++e)
-        h[e] = v8 + e < V ? __float_as_uint(__ldg(row + v8 + e)) : ninf;
-      w[0] = make_uint4(h[0], h[1], h[2], h[3]);
-      w[1] = make_uint4(h[4], h[5], h[6], h[7]);
-    }
-  }
-  __device__ static void unpack(const uint4 (&w)[kWords], float (&x)[8]) {
-    x[0] = __uint_as_float(w[0].x), x[1] = __uint_as_float(w[0].y), x[2] = __uint_as_float(w[0].z);
-    x[3] = __uint_as_float(w[0].w), x[4] = __uint_as_float(w[1].x), x[5] = __uint_as_float(w[1].y);
-    x[6] = __uint_as_float(w[1].z), x[7] = __uint_as_float(w[1].w);
-  }
-  template <int N>
-  __device__ static float round_max(const uint4 (&w)[N][kWords]) {
-    float m[N];
-#pragma unroll
-    for (int u = 0; u < N; ++u) {
-      float x[8];
-      unpack(w[u], x);
-      m[u] = fmaxf(fmaxf(fmaxf(x[0], x[1]), fmaxf(x[2], x[3])), fmaxf(fmaxf(x[4], x[5]), fmaxf(x[6], x[7])));
-    }
-#pragma unroll
-    for (int n = N / 2; n > 0; n >>= 1)
-#pragma unroll
-      for (int u = 0; u < n; ++u) m[u] = fmaxf(m[u], m[u + n]);
-    return m[0];
-  }
+struct Round<float> {
+  static constexpr int kBlocks = 4;
+  static constexpr int kHalf = 1;
+  static constexpr int kLines = 8;
+  static constexpr int kPer = 4;
+  static constexpr uint32_t kPad = 0xFF800000u;
 };
 
-// Per-warp state of a chunk (identical in every lane).
+// First entry of word u of lane l in the round that starts at block b0.
+template <typename T>
+__device__ __forceinline__ int word_entry(int b0, int u, int lane) {
+  using R = Round<T>;
+  return (b0 + 4 * (u / R::kLines) + (lane >> 3)) * kRaceBlock + (u % R::kLines) * (8 * R::kPer) + (lane & 7) * R::kPer;
+}
+
+// 16 bytes of a row at entry v from any alignment: the two aligned words that
+// hold them, shifted together.  A word is read only if it lies inside the
+// logits [lo, hi); at their two ends, and where fewer than a word's entries
+// are left, the entries are read one by one (past vend: -inf).
+template <typename T>
+__device__ __forceinline__ uint4 load_shifted(const T* row, int v, int vend, uintptr_t lo, uintptr_t hi) {
+  using R = Round<T>;
+  const uint32_t pad = R::kPad;
+  if (v >= vend) return make_uint4(pad, pad, pad, pad);
+  const uintptr_t a = reinterpret_cast<uintptr_t>(row + v);
+  const uintptr_t w0 = a & ~(uintptr_t)15;
+  if (v + R::kPer <= vend && w0 >= lo && w0 + 32 <= hi) {
+    const uint4 x = __ldg(reinterpret_cast<const uint4*>(w0)), y = __ldg(reinterpret_cast<const uint4*>(w0) + 1);
+    const uint32_t s = (uint32_t)(a & 15u), bits = 8u * (s & 3u);
+    // drop s bytes of the 32: whole words by selection, the rest by a funnel shift
+    const uint32_t in[8] = {x.x, x.y, x.z, x.w, y.x, y.y, y.z, y.w};
+    uint32_t t[5];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+      const uint32_t p = s < 4 ? in[k] : in[k + 1], q = s < 12 ? in[k + 2] : in[k + 3 > 7 ? 7 : k + 3];
+      t[k] = s < 8 ? p : q;
+    }
+    return make_uint4(__funnelshift_r(t[0], t[1], bits), __funnelshift_r(t[1], t[2], bits),
+                      __funnelshift_r(t[2], t[3], bits), __funnelshift_r(t[3], t[4], bits));
+  }
+  uint32_t h[8];
+#pragma unroll
+  for (int e = 0; e < R::kPer; ++e) {
+    if (sizeof(T) == 4)
+      h[e] = v + e < vend ? __float_as_uint(__ldg(reinterpret_cast<const float*>(row) + v + e)) : pad;
+    else
+      h[e] = v + e < vend ? (uint32_t)__ldg(reinterpret_cast<const unsigned short*>(row) + v + e) : 0xFF80u;
+  }
+  if (sizeof(T) == 4) return make_uint4(h[0], h[1], h[2], h[3]);
+  return make_uint4(h[0] | h[1] << 16, h[2] | h[3] << 16, h[4] | h[5] << 16, h[6] | h[7] << 16);
+}
+
+// The round's words (entries at or past vend read -inf).
+template <typename T, bool kVec>
+__device__ __forceinline__ void load_round(uint4 (&w)[8], const T* row, int b0, int vend, int lane, uintptr_t lo,
+                                           uintptr_t hi) {
+  using R = Round<T>;
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const int v = word_entry<T>(b0, u, lane);
+    if (kVec) w[u] = v < vend ? ldg_stream(row + v) : make_uint4(R::kPad, R::kPad, R::kPad, R::kPad);
+    else w[u] = load_shifted(row, v, vend, lo, hi);
+  }
+}
+
+// Max over a lane's words (a NaN loses to any number here; the sums catch it).
+__device__ __forceinline__ float words_max(const uint4 (&w)[8], __nv_bfloat16) {
+  __nv_bfloat162 m[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) {
+    const __nv_bfloat162* h = reinterpret_cast<const __nv_bfloat162*>(&w[u]);
+    m[u] = __hmax2(__hmax2(h[0], h[1]), __hmax2(h[2], h[3]));
+  }
+#pragma unroll
+  for (int n = 4; n > 0; n >>= 1)
+#pragma unroll
+    for (int u = 0; u < n; ++u) m[u] = __hmax2(m[u], m[u + n]);
+  return fmaxf(__low2float(m[0]), __high2float(m[0]));
+}
+__device__ __forceinline__ float words_max(const uint4 (&w)[8], float) {
+  float m[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    m[u] = fmaxf(fmaxf(__uint_as_float(w[u].x), __uint_as_float(w[u].y)),
+                 fmaxf(__uint_as_float(w[u].z), __uint_as_float(w[u].w)));
+#pragma unroll
+  for (int n = 4; n > 0; n >>= 1)
+#pragma unroll
+    for (int u = 0; u < n; ++u) m[u] = fmaxf(m[u], m[u + n]);
+  return m[0];
+}
+
+// A warp's running state over its segment.  m (and at tau = 0 first) is the
+// same in every lane; s and best are the lane's own parts.
 struct WarpDraftState {
-  SoftState st{-INFINITY, 0.0f};
-  BlockKey best{INFINITY, 0.0f, INT_MAX};  // tau > 0
-  ArgState g{-INFINITY, INT_MAX};          // tau = 0: (max, lowest index)
-  int32_t flags = 0;
+  float m = -INFINITY, s = 0.0f;           // max, and the lane's sum of 2^(l*c2 - fl(m*c2)); NaN once a NaN or +inf was read
+  BlockKey best{INFINITY, 0.0f, INT_MAX};  // tau > 0: the best of the lane's blocks
+  int32_t first = INT_MAX;                 // tau = 0: first block of the first round that reaches m
+  float keep_s = 0.0f, keep_m = 0.0f;      // tau > 0: the lane's block of the current 32: its sum, relative to keep_m
 };
 
-// Sum of per-lane values acc[u] (u < N, N = 4 or 8: one per race block of
-// the round) over the warp, transposed: after log2 N halving exchanges and a
-// butterfly over the remaining lane bits, lane l holds the sum of block
-// l >> (5 - log2 N); the 32 / N lanes of a block hold identical values.
-template <int N>
-__device__ __forceinline__ float transposed_block_sum(const float (&acc)[N], int lane) {
-  static_assert(N == 4 || N == 8, "4 or 8 blocks per round");
-  float v[N];
-#pragma unroll
-  for (int u = 0; u < N; ++u) v[u] = acc[u];
-#pragma unroll
-  for (int n = N, o = 16; n > 1; n >>= 1, o >>= 1) {
-    const bool hi = (lane & o) != 0;
-#pragma unroll
-    for (int j = 0; j < n / 2; ++j) {
-      const float send = hi ? v[j] : v[j + n / 2];
-      const float keep = hi ? v[j + n / 2] : v[j];
-      v[j] = keep + __shfl_xor_sync(0xFFFFFFFFu, send, o);
-    }
-  }
-#pragma unroll
-  for (int o = 16 / N; o > 0; o >>= 1) v[0] += __shfl_xor_sync(0xFFFFFFFFu, v[0], o);
-  return v[0];
+// The lane's block among each 32 (level 1 of the race): the round whose index
+// in the 32 equals owned_round(), and in it the block whose sum block_sum()
+// leaves in the lane.
+template <typename T>
+__device__ __forceinline__ int owned_round(int lane) { return lane & (Round<T>::kHalf == 2 ? 3 : 7); }
+template <typename T>
+__device__ __forceinline__ int owned_block(int lane) {
+  return Round<T>::kHalf == 2 ? 8 * (lane & 3) + (lane & 4) + (lane >> 3) : 4 * (lane & 7) + (lane >> 3);
+}
+// Sum over the block's 8 lanes: with two blocks per lane group, lanes with bit
+// 2 set end with the second one's.
+__device__ __forceinline__ float block_sum(const float (&acc)[2], int lane) {
+  const bool hi = (lane & 4) != 0;
+  float v = (hi ? acc[1] : acc[0]) + __shfl_xor_sync(0xFFFFFFFFu, hi ? acc[0] : acc[1], 4);
+  v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+  return v + __shfl_xor_sync(0xFFFFFFFFu, v, 1);
+}
+__device__ __forceinline__ float block_sum(const float (&acc)[1], int) {
+  float v = acc[0] + __shfl_xor_sync(0xFFFFFFFFu, acc[0], 4);
+  v += __shfl_xor_sync(0xFFFFFFFFu, v, 2);
+  return v + __shfl_xor_sync(0xFFFFFFFFu, v, 1);
 }
 
-// soft_merge with the scale factor from ex2.approx (relative error ~2^-22):
-// the per-round merges of the streaming softmax.
-__device__ __forceinline__ SoftState soft_merge_fast(SoftState a, SoftState b, float c2) {
-  if (b.m > a.m) {
-    const SoftState t = a;
-    a = b;
-    b = t;
-  }
-  if (b.m == -INFINITY) return a;
-  a.s = a.s + b.s * ex2_approx(b.m * c2 - a.m * c2);
-  return a;
-}
-
-// The level-1 race words of blocks g0 .. g0+31 (g0 a multiple of 32), lane
-// l holding block g0 + l's: word l & 3 of the Philox quad at counter
-// (g0 >> 2) + (l >> 2).  One quad per lane serves 32 / N rounds.
-__device__ __forceinline__ uint32_t race_words(int g0, int lane, uint32_t position, uint64_t req, uint32_t k0,
-                                               uint32_t k1) {
-  const uint4 rq = philox(draw_counter(position, req, SPEC_PURPOSE_DRAFT, (uint32_t)((g0 >> 2) + (lane >> 2))), k0, k1);
-  const int e = lane & 3;
+// The level-1 race word of the lane's block among blocks g0 .. g0+31 (g0 a
+// multiple of 32): word l >> 3 of the Philox quad of blocks
+// g0 + (owned_block & ~3) .. +3.
+template <typename T>
+__device__ __forceinline__ uint32_t race_word(int g0, int lane, uint32_t position, uint64_t req, uint32_t k0,
+                                              uint32_t k1) {
+  const uint4 rq =
+      philox(draw_counter(position, req, SPEC_PURPOSE_DRAFT, (uint32_t)((g0 + owned_block<T>(lane)) >> 2)), k0, k1);
+  const int e = lane >> 3;
   return e == 0 ? rq.x : e == 1 ? rq.y : e == 2 ? rq.z : rq.w;
 }
 
-// One round of N consecutive race blocks b0 .. b0+N-1 of the warp (blocks at
-// or past b_hi were loaded as -inf).  Every value is taken relative to the
-// round's max M_r: the blocks' sums of 2^(l*c2 - fl(M_r*c2)) (a block whose
-// weight underflows against M_r is more than 2^-126 below the round's best
-// and cannot win the race), the round's softmax contribution, and each
-// block's level-1 candidate (L = log2 E_b - log2 sum_b, M = M_r), one block
-// per lane group.  Lane l's `rword` is the race word of block g0 + l, g0 the
-// first block of the group of 32 that holds this round (race_words).
+// One round of consecutive race blocks from b0.  Every value is taken relative
+// to the round's max M_r: a block whose weight underflows against M_r is more
+// than 2^-126 below the round's best and cannot win the race.  A NaN or a +inf
+// entry makes the lane's sum NaN, which stays; a round of -inf adds 0.
 template <typename T, bool kGreedy>
-__device__ __forceinline__ void draft_round(WarpDraftState& ws, const uint4 (&w)[Lane8<T>::kBlocksPerRound][Lane8<T>::kWords],
-                                            int b0, int b_hi, int lane, float c2, uint32_t rword) {
-  using L8 = Lane8<T>;
-  constexpr int N = L8::kBlocksPerRound;
-  // ---- the round's max (+inf makes the row unusable; a NaN is caught by
-  // the sums below, which it turns into NaN) ----
-  const float lmax = L8::template round_max<N>(w);
-  const float Mr = from_orderable(__reduce_max_sync(0xFFFFFFFFu, orderable(lmax)));
-  if (Mr == INFINITY) {
-    ws.flags |= 1;
-    return;
-  }
-  if (Mr == -INFINITY) {  // no finite entry in the round: weight 0, unless a NaN hides here
-    bool nan = false;
-#pragma unroll
-    for (int u = 0; u < N; ++u) {
-      float x[8];
-      L8::unpack(w[u], x);
-#pragma unroll
-      for (int e = 0; e < 8; ++e) nan |= x[e] != x[e];
-    }
-    if (__any_sync(0xFFFFFFFFu, nan)) ws.flags |= 1;
-    return;
-  }
-  if (kGreedy && (ws.g.idx == INT_MAX || Mr > ws.g.v)) {
-    // a new running max: its first index (rounds arrive in increasing order)
-    unsigned first = 0xFFFFFFFFu;
-#pragma unroll
-    for (int u = N - 1; u >= 0; --u) {
-      float x[8];
-      L8::unpack(w[u], x);
-#pragma unroll
-      for (int e = 7; e >= 0; --e)
-        if (x[e] == Mr) first = (unsigned)((b0 + u) * kRaceBlock + 8 * lane + e);
-    }
-    ws.g = ArgState{Mr, (int)__reduce_min_sync(0xFFFFFFFFu, first)};
-  }
-  // ---- per-block sums relative to the round's max ----
-  const float M2 = Mr * c2;
+__device__ __forceinline__ void draft_round(WarpDraftState& ws, const uint4 (&w)[8], int b0, int lane, float c2) {
+  using R = Round<T>;
+  const float Mr = from_orderable(__reduce_max_sync(0xFFFFFFFFu, orderable(words_max(w, T()))));
+  const float M2 = Mr > -INFINITY ? Mr * c2 : 0.0f;
   const float2 c2v = make_float2(c2, c2), nM2 = make_float2(-M2, -M2);
-  float acc[N];
+  float acc[R::kHalf];
 #pragma unroll
-  for (int u = 0; u < N; ++u) {
-    float x[8];
-    L8::unpack(w[u], x);
+  for (int h = 0; h < R::kHalf; ++h) {
     float2 a0 = make_float2(0.f, 0.f), a1 = make_float2(0.f, 0.f);
 #pragma unroll
-    for (int e = 0; e < 8; e += 4) {
-      const float2 y0 = __ffma2_rn(make_float2(x[e], x[e + 1]), c2v, nM2);
-      const float2 y1 = __ffma2_rn(make_float2(x[e + 2], x[e + 3]), c2v, nM2);
-      a0 = __fadd2_rn(a0, make_float2(ex2_approx(y0.x), ex2_approx(y0.y)));
-      a1 = __fadd2_rn(a1, make_float2(ex2_approx(y1.x), ex2_approx(y1.y)));
-    }
-    acc[u] = (a0.x + a0.y) + (a1.x + a1.y);
-  }
-  const int ub = lane >> (N == 8 ? 2 : 3);  // this lane's block of the round
-  const float sb = transposed_block_sum<N>(acc, lane);
-  float sr = sb;  // the round's sum: add the N distinct blocks
+    for (int l = 0; l < R::kLines; ++l) {
 #pragma unroll
-  for (int o = 32 / N; o < 32; o <<= 1) sr += __shfl_xor_sync(0xFFFFFFFFu, sr, o);
-  if (sr != sr) {  // a NaN entry
-    ws.flags |= 1;
-    return;
+      for (int e = 0; e < R::kPer; e += 4) {
+        const uint4& x = w[h * R::kLines + l];
+        const float2 y0 = __ffma2_rn(make_float2(Vec<T>::get(x, e), Vec<T>::get(x, e + 1)), c2v, nM2);
+        const float2 y1 = __ffma2_rn(make_float2(Vec<T>::get(x, e + 2), Vec<T>::get(x, e + 3)), c2v, nM2);
+        a0 = __fadd2_rn(a0, make_float2(ex2_approx(y0.x), ex2_approx(y0.y)));
+        a1 = __fadd2_rn(a1, make_float2(ex2_approx(y1.x), ex2_approx(y1.y)));
+      }
+    }
+    acc[h] = (a0.x + a0.y) + (a1.x + a1.y);
   }
-  ws.st = soft_merge_fast(ws.st, SoftState{Mr, sr}, c2);
+  // the softmax state: the lane's part, scaled to the larger max
+  const float own = R::kHalf == 2 ? acc[0] + acc[R::kHalf - 1] : acc[0];
+  if (Mr > ws.m) {
+    ws.s = fmaf(ws.s, ex2_approx(ws.m * c2 - M2), own);
+    ws.m = Mr;
+    if (kGreedy) ws.first = b0;
+  } else {
+    ws.s = Mr > -INFINITY ? fmaf(own, ex2_approx(M2 - ws.m * c2), ws.s) : ws.s + own;
+  }
   if (kGreedy) return;
-  // ---- level-1 candidates, one block per lane group ----
-  const int b = b0 + ub;
-  const uint32_t word = __shfl_sync(0xFFFFFFFFu, rword, b & 31);
+  const float sb = block_sum(acc, lane);
+  if (((b0 & (kGroup - 1)) / R::kBlocks) == owned_round<T>(lane)) {
+    ws.keep_s = sb;
+    ws.keep_m = Mr;
+  }
+}
+
+// Level-1 key of the lane's block `b` once its round is in (b < b_hi).
+__device__ __forceinline__ void draft_candidate(WarpDraftState& ws, int b, uint32_t word, float c2) {
   // E near 0 needs log1pf; log2 of E and of the sum go to lg2.approx, whose
   // absolute error (~1e-7) is what a log-domain key can afford
-  KeyState cand{INFINITY, INT_MAX};
-  if (b < b_hi && sb > 0.0f) {
-    const float E = -log1pf(-((float)race_m(word) * 0x1p-24f));
-    cand = KeyState{lg2_approx(E) - lg2_approx(sb), b};
-  }
-  // every candidate of the round shares M = M_r: compare L alone
-#pragma unroll
-  for (int o = 32 / N; o < 32; o <<= 1) {
-    const KeyState other{__shfl_xor_sync(0xFFFFFFFFu, cand.key, o), __shfl_xor_sync(0xFFFFFFFFu, cand.idx, o)};
-    if (key_better(other, cand)) cand = other;
-  }
-  if (cand.idx != INT_MAX) {
-    const BlockKey rb{cand.key, Mr, cand.idx};
-    if (block_key_better(rb, ws.best, c2)) ws.best = rb;
-  }
+  if (!(ws.keep_s > 0.0f)) return;
+  const float E = -log1pf(-((float)race_m(word) * 0x1p-24f));
+  const BlockKey k{lg2_approx(E) - lg2_approx(ws.keep_s), ws.keep_m, b};
+  if (block_key_better(k, ws.best, c2)) ws.best = k;
 }
 
 // Minimum key over the warp (every lane).
@@ -361,66 +339,84 @@ __device__ __forceinline__ KeyState warp_min_key(KeyState b) {
   return b;
 }
 
-// One warp per (row, segment of SB blocks); the warps of a CTA are
-// independent (no CTA barrier).  The last warp of a row to arrive merges the
-// row's segment partials, draws inside the winning block and writes the
-// row's outputs; the last row of a request writes the scores.
+// One warp per (row, segment of blocks); the warps of a CTA are independent
+// (no CTA barrier).  The last warp of a row to arrive merges the row's segment
+// partials, draws inside the winning block and writes the row's outputs; the
+// last row of a request writes the scores.
 template <typename T, bool kGreedy, bool kVec>
-__global__ void __launch_bounds__(kDraftThreads, 4) draft_rows_kernel(const DraftLaunch p) {
+__global__ void __launch_bounds__(kDraftThreads, kDraftCtas) draft_rows_kernel(const DraftLaunch p) {
+  using R = Round<T>;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const long long unit = (long long)blockIdx.x * (kDraftThreads / 32) + warp;
-  pdl_wait_prerequisites();
-  pdl_launch_dependents();
   if (unit >= (long long)p.B * p.K * p.NC) return;
   const int r = (int)(unit / p.NC);
   const int c = (int)(unit - (long long)r * p.NC);
   const int i = r / p.K;
   const int k = r - i * p.K;
   const T* row = static_cast<const T*>(p.logits) + (size_t)r * (size_t)p.V;
+  const uintptr_t lo = reinterpret_cast<uintptr_t>(p.logits);
+  const uintptr_t hi = lo + (size_t)p.B * p.K * (size_t)p.V * sizeof(T);
 
   // ---- this segment's blocks, a round of consecutive ones at a time ----
   const int nb = (p.V + kRaceBlock - 1) / kRaceBlock;
   const int bps = p.chunk / kRaceBlock;
   const int b_lo = c * bps, b_hi = min(nb, b_lo + bps);
-  using L8 = Lane8<T>;
-  constexpr int kBPR = L8::kBlocksPerRound;
-  uint4 w[kBPR][L8::kWords];
-  auto load_round = [&](int b0) {
-#pragma unroll
-    for (int u = 0; u < kBPR; ++u)
-      L8::template load<kVec>(row, (b0 + u) * kRaceBlock + 8 * lane, b0 + u < b_hi ? p.V : 0, w[u]);
-  };
-  if (b_lo < b_hi) load_round(b_lo);  // the first loads ahead of the request's scalars
+  const int vend = (int)min((long long)p.V, (long long)b_hi * kRaceBlock);
+  // The segment's first round starts towards L2 (a line a lane) while the
+  // previous kernel on the stream drains: a prefetch returns no data, and L2
+  // is where that kernel's writes arrive, so nothing is read early.
+  const int v_pre = b_lo * kRaceBlock + lane * (128 / (int)sizeof(T));
+  if (v_pre < vend) asm volatile("prefetch.global.L2 [%0];" ::"l"(row + v_pre));
+  pdl_wait_prerequisites();
+  pdl_launch_dependents();
+  uint4 w[8];
+  load_round<T, kVec>(w, row, b_lo, vend, lane, lo, hi);  // the first loads ahead of the request's scalars
   const long long pos = __ldg(reinterpret_cast<const long long*>(p.pos_base) + i);
-  const bool pos_ok = pos >= 0 && pos + p.K <= 0xFFFFFFFFLL;
   const uint32_t position = (uint32_t)(pos + k + 1);
   const uint64_t req = __ldg(reinterpret_cast<const unsigned long long*>(p.request_ids) + i);
   const uint64_t seed = __ldg(reinterpret_cast<const unsigned long long*>(p.seeds) + i);
   const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
   WarpDraftState ws;
-  uint32_t rword = 0;
-  for (int b0 = b_lo; b0 < b_hi; b0 += kBPR) {
-    if (b0 != b_lo) load_round(b0);
-    if (!kGreedy && (b0 == b_lo || (b0 & 31) == 0)) rword = race_words(b0 & ~31, lane, position, req, k0, k1);
-    draft_round<T, kGreedy>(ws, w, b0, b_hi, lane, p.c2, rword);
+  uint32_t word = 0;
+  for (int b0 = b_lo; b0 < b_hi; b0 += R::kBlocks) {
+    if (b0 != b_lo) load_round<T, kVec>(w, row, b0, vend, lane, lo, hi);
+    // the group's race words, drawn while the loads are in flight
+    if (!kGreedy && (b0 == b_lo || (b0 & (kGroup - 1)) == 0)) {
+      word = race_word<T>(b0 & ~(kGroup - 1), lane, position, req, k0, k1);
+      ws.keep_s = 0.0f;
+    }
+    draft_round<T, kGreedy>(ws, w, b0, lane, p.c2);
+    const int bn = b0 + R::kBlocks;
+    if (!kGreedy && (bn >= b_hi || (bn & (kGroup - 1)) == 0))
+      draft_candidate(ws, (b0 & ~(kGroup - 1)) + owned_block<T>(lane), word, p.c2);
   }
 
-  // ---- the segment's partial; the last warp of the row goes on ----
+  // ---- the segment's partial over the lanes; the last warp of the row goes on ----
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) {
+    ws.s += __shfl_xor_sync(0xFFFFFFFFu, ws.s, o);
+    if (!kGreedy) {
+      const BlockKey ob{__shfl_xor_sync(0xFFFFFFFFu, ws.best.L, o), __shfl_xor_sync(0xFFFFFFFFu, ws.best.M, o),
+                        __shfl_xor_sync(0xFFFFFFFFu, ws.best.idx, o)};
+      if (block_key_better(ob, ws.best, p.c2)) ws.best = ob;
+    }
+  }
   int last = 0;
   if (lane == 0) {
     DraftPartial d{};
-    d.m = ws.st.m;
-    d.s = ws.st.s;
-    d.key = kGreedy ? ws.g.v : ws.best.L;
+    d.m = ws.m;
+    d.s = ws.s;
+    d.key = kGreedy ? ws.m : ws.best.L;
     d.keyM = kGreedy ? 0.0f : ws.best.M;
-    d.idx = kGreedy ? ws.g.idx : ws.best.idx;
-    d.flags = ws.flags;
+    d.idx = kGreedy ? ws.first : ws.best.idx;
+    d.flags = ws.s != ws.s;
     p.part[(size_t)r * p.NC + c] = d;
     __threadfence();  // the partial before the count
     last = atomicAdd(p.row_count + r, 1u) == (uint32_t)(p.NC - 1);
   }
   if (!__shfl_sync(0xFFFFFFFFu, last, 0)) return;
   __threadfence();  // the other segments' partials after their counts
+  const bool pos_ok = pos >= 0 && pos + p.K <= 0xFFFFFFFFLL;
 
   // ---- merge the row's segments (lanes over segments) ----
   SoftState st{-INFINITY, 0.0f};
@@ -458,7 +454,16 @@ __global__ void __launch_bounds__(kDraftThreads, 4) draft_rows_kernel(const Draf
   int z = -1;
   if (!bad) {
     if (kGreedy) {
-      z = idx;
+      // the first entry of the round from block idx that equals the max
+      load_round<T, kVec>(w, row, idx, p.V, lane, lo, hi);
+      unsigned first = 0xFFFFFFFFu;
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+#pragma unroll
+        for (int e = 0; e < R::kPer; ++e)
+          if (Vec<T>::get(w[u], e) == st.m) first = min(first, (unsigned)(word_entry<T>(idx, u, lane) + e));
+      first = __reduce_min_sync(0xFFFFFFFFu, first);
+      z = first == 0xFFFFFFFFu ? -1 : (int)first;
     } else {
       // level 2 in the winning block (8 entries per lane), weights relative
       // to the row max
@@ -484,45 +489,60 @@ __global__ void __launch_bounds__(kDraftThreads, 4) draft_rows_kernel(const Draf
       z = e.idx == INT_MAX ? -1 : e.idx;
     }
   }
-  if (lane != 0) return;
-  const size_t o = (size_t)i * p.K + k;
-  if (bad || z < 0) {
-    p.drafts[o] = -1;
-    p.conf[o] = 0.0f;
-    if (p.row_stats) reinterpret_cast<float2*>(p.row_stats)[o] = make_float2(0.0f, 0.0f);
-    atomicOr(p.req_bad + i, 1u);
-  } else {
-    p.drafts[o] = z;
-    // c = q(z) = 2^(l_z*c2 - fl(m*c2)) / S, with one rounding in the exponent
-    p.conf[o] = exp2f(fmaf(load_elem(row + z), p.c2, -M2)) / st.s;
-    if (p.row_stats) {
-      const float resid = fmaf(st.m, p.c2, -M2);
-      reinterpret_cast<float2*>(p.row_stats)[o] = make_float2(st.m * p.inv_t, (log2f(st.s) - resid) * 0.69314718055994531f);
+  int last_row = 0;
+  if (lane == 0) {
+    const size_t o = (size_t)i * p.K + k;
+    if (bad || z < 0) {
+      p.drafts[o] = -1;
+      p.conf[o] = 0.0f;
+      if (p.row_stats) reinterpret_cast<float2*>(p.row_stats)[o] = make_float2(0.0f, 0.0f);
+      atomicOr(p.req_bad + i, 1u);
+    } else {
+      p.drafts[o] = z;
+      // c = q(z) = 2^(l_z*c2 - fl(m*c2)) / S, with one rounding in the exponent
+      p.conf[o] = exp2f(fmaf(load_elem(row + z), p.c2, -M2)) / st.s;
+      if (p.row_stats) {
+        const float resid = fmaf(st.m, p.c2, -M2);
+        reinterpret_cast<float2*>(p.row_stats)[o] = make_float2(st.m * p.inv_t, (log2f(st.s) - resid) * 0.69314718055994531f);
+      }
     }
+    __threadfence();  // this row's outputs before the count
+    last_row = atomicAdd(p.req_count + i, 1u) == (uint32_t)(p.K - 1);
   }
-  // ---- the last row of the request: the scores ----
-  __threadfence();  // this row's outputs before the count
-  if (atomicAdd(p.req_count + i, 1u) != (uint32_t)(p.K - 1)) return;
+  // ---- the last row of the request: the scores, the warp loading 32
+  // confidences at a time and multiplying them in order ----
+  if (!__shfl_sync(0xFFFFFFFFu, last_row, 0)) return;
   __threadfence();
-  p.req_count[i] = 0u;
   const bool req_bad = __ldcg(p.req_bad + i) != 0u;
-  if (req_bad) {
-    p.req_bad[i] = 0u;
-    report(p.status, SPEC_ERR_BAD_INPUT);
-    for (int kk = 0; kk < p.K; ++kk) {
-      p.drafts[(size_t)i * p.K + kk] = -1;
-      p.conf[(size_t)i * p.K + kk] = 0.0f;
-      if (p.row_stats) reinterpret_cast<float2*>(p.row_stats)[(size_t)i * p.K + kk] = make_float2(0.0f, 0.0f);
+  __syncwarp();  // every lane has read the flag
+  if (lane == 0) {
+    p.req_count[i] = 0u;
+    if (req_bad) {
+      p.req_bad[i] = 0u;
+      report(p.status, SPEC_ERR_BAD_INPUT);
     }
   }
-  if (p.scores) {
-    float* sc = p.scores + (size_t)i * (p.K + 1);
-    float run = 1.0f;
-    sc[0] = run;
-    for (int kk = 0; kk < p.K; ++kk) {
-      run = req_bad ? 0.0f : __fmul_rn(run, __ldcg(p.conf + (size_t)i * p.K + kk));
-      sc[kk + 1] = run;
+  float run = 1.0f;
+  if (p.scores && lane == 0) p.scores[(size_t)i * (p.K + 1)] = run;
+  for (int base = 0; base < p.K; base += 32) {
+    const int kk = base + lane;
+    const size_t o = (size_t)i * p.K + kk;
+    float cf = 0.0f, mine = 0.0f;
+    if (kk < p.K) {
+      if (req_bad) {
+        p.drafts[o] = -1;
+        p.conf[o] = 0.0f;
+        if (p.row_stats) reinterpret_cast<float2*>(p.row_stats)[o] = make_float2(0.0f, 0.0f);
+      } else {
+        cf = __ldcg(p.conf + o);
+      }
     }
+    const int n = min(32, p.K - base);
+    for (int j = 0; j < n; ++j) {
+      run = __fmul_rn(run, __shfl_sync(0xFFFFFFFFu, cf, j));
+      if (lane == j) mine = run;
+    }
+    if (p.scores && kk < p.K) p.scores[(size_t)i * (p.K + 1) + kk + 1] = mine;
   }
 }
 

@@ -171,3 +171,33 @@ def test_draft_to_allocation():
     ga = gpu_allocate(conf, Ts, costs)
     ra = oracle.allocate(g["c"], Ts, costs)
     assert_alloc_equal(ga, ra)
+
+
+@pytest.mark.parametrize("dtype,offset", [("bf16", o) for o in range(1, 8)] + [("f32", o) for o in range(1, 4)])
+@pytest.mark.parametrize("V", [2049, 4096])
+def test_every_alignment(dtype, offset, V):
+    """Rows at every offset from a 16-byte boundary (two aligned words shifted
+    together): odd V moves the offset from row to row, even V keeps it.  The
+    words at the tensor's ends are read entry by entry, with the guard entries
+    around it (+inf, which would mark the row) never taken in."""
+    x, seeds, rids, pos = _case(3, 4, V, dtype, V + offset)
+    buf = torch.full((x.numel() + 16,), float("inf"), dtype=x.dtype, device=DEV)
+    view = buf[offset:offset + x.numel()].view(x.shape)
+    view.copy_(x.to(DEV))
+    for tau in (0.0, 0.8):
+        g = run_draft(view, tau, seeds, rids, pos)
+        assert g["status"] == 0
+        compare_draft(g, run_oracle_draft(x, tau, seeds, rids, pos), tau)
+
+
+# Segments of 16, 24 and 32 blocks (8 in the small shapes above), so that a
+# segment starts inside a group of 32 race blocks, with a short last round; and
+# ties of the row's max within a round, a segment and across segments.
+@pytest.mark.parametrize("B,K,V,dtype", [(8, 8, 170001, "bf16"), (16, 8, 204792, "bf16"), (32, 8, 131080, "bf16"),
+                                         (8, 8, 170004, "f32"), (16, 8, 204799, "f32")])
+@pytest.mark.parametrize("tau", [0.0, 1.0])
+def test_segment_lengths(B, K, V, dtype, tau):
+    x, seeds, rids, pos = _case(B, K, V, dtype, V)
+    if tau == 0.0:
+        x = (x * 2).round() / 2  # few values: every row's max is tied many times
+    compare_draft(run_draft(x, tau, seeds, rids, pos), run_oracle_draft(x, tau, seeds, rids, pos), tau)
