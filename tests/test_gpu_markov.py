@@ -203,3 +203,40 @@ def test_batches_past_the_repeated_rows_and_three_atom_rank(B, r):
     o = run_oracle_markov(U, W1, W2, x0, 0.9, seeds, rids, pos)
     assert g["status"] == 0 and (o["status"] == 0).all()
     assert compare_markov(g, o, U, W1, W2, x0, 0.9) <= max(1, B // 32)
+
+
+# The bias kernel's ways of reading U: whole tiles through the tensor map with
+# one request copy per lane half (B <= 64, at most and above 32), column halves
+# (B > 64), one to three units in flight (r = 256, 192, 64); V a multiple of 8
+# that ends inside a sub-block, inside the first half of a tile, at a tile's
+# end and below one sub-block, with more tiles than SMs; and direct loads for
+# other V.
+@pytest.mark.parametrize("B", [2, 40, 64, 65, 128])
+@pytest.mark.parametrize("V,r", [(56, 64), (2568, 256), (2688, 192), (1000, 64), (21000, 256), (40008, 64), (21001, 128)])
+@pytest.mark.parametrize("tau", [0.0, 1.0])
+def test_bias_tiles(B, V, r, tau):
+    U, W1, W2, x0, seeds, rids, pos = _case(B, 2, V, r, 3 * V + B)
+    g = run_markov(U, W1, W2, x0, tau, seeds, rids, pos)
+    assert g["status"] == 0
+    some = sorted({0, 1, B // 2, B - 1})
+    o = run_oracle_markov(U, W1, W2, x0, tau, seeds, rids, pos, requests=some)
+    assert compare_markov(g, o, U, W1, W2, x0, tau, requests=some) <= 1
+
+
+@pytest.mark.parametrize("V", [2568, 2567])
+@pytest.mark.parametrize("value", [float("nan"), float("inf")])
+def test_bad_entries_in_any_tile(V, value):
+    """A NaN or +inf anywhere in a request's U (also among -inf entries) marks
+    that request and no other."""
+    B = 6
+    U, W1, W2, x0, seeds, rids, pos = _case(B, 2, V, 64, 99)
+    U[1, 0, 0] = value
+    U[2, 1, V - 1] = value
+    U[4, 0, 64:128] = float("-inf")
+    U[4, 0, 100] = value
+    U[5, 0, 64:256] = float("-inf")  # allowed: no weight there
+    for tau in (0.0, 1.0):
+        g = run_markov(U, W1, W2, x0, tau, seeds, rids, pos)
+        assert (g["z"] == -1).all(axis=1).tolist() == [False, True, True, False, True, False]
+        o = run_oracle_markov(U, W1, W2, x0, tau, seeds, rids, pos)
+        compare_markov(g, o, U, W1, W2, x0, tau)
