@@ -9,6 +9,7 @@ Round of arxiv 2607.25852 (AngelSpec): ``spec_allocate`` (D-cut, Section 4.2)
 -> target forward over the packed rows (caller) -> ``spec_verify`` (rejection
 sampling, Section 1) -> ``spec_commit`` (packing for the next drafting step).
 """
+import array
 import ctypes
 
 import torch
@@ -54,33 +55,60 @@ class SpecError(RuntimeError):
 
 def library():
     """The loaded ctypes handle of libspec.so."""
-    return _native.load()
+    return _native._lib or _native.load()
+
+
+# The helpers below run for every argument of every call, and a round's small
+# calls cost the host more than the GPU: addresses go to ctypes as plain
+# integers (its declared argument types convert them), and the current stream
+# comes from torch's raw-handle query (0.2 us; building a torch Stream object
+# took 3.1 us of a 16 us spec_verify call).
+_DTYPES = {torch.bfloat16: BF16, torch.float32: F32}
+_Tensor = torch.Tensor
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)  # absent from CPU-only builds
+_current_device = getattr(torch._C, "_cuda_getDevice", None)
 
 
 def _ptr(t):
     if t is None:
         return None
-    if not isinstance(t, torch.Tensor):
+    if not isinstance(t, _Tensor):
         raise TypeError("expected a torch.Tensor or None")
     if not t.is_contiguous():
         raise ValueError("tensors passed to libspec must be contiguous")
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
 
 
 def _dtype(t):
     if t is None:
         return BF16
-    if t.dtype == torch.bfloat16:
-        return BF16
-    if t.dtype == torch.float32:
-        return F32
-    raise TypeError(f"unsupported element type {t.dtype} (bf16 or fp32)")
+    code = _DTYPES.get(t.dtype)
+    if code is None:
+        raise TypeError(f"unsupported element type {t.dtype} (bf16 or fp32)")
+    return code
 
 
 def _stream(stream):
     if stream is None:
+        if _raw_stream is not None and torch.cuda.is_initialized():
+            return _raw_stream(_current_device())
         stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    return stream.cuda_stream
+
+
+def _int32s(xs):
+    """Host int32s for a C call: an array.array, its address in buffer_info()."""
+    try:
+        return array.array("i", xs)
+    except (TypeError, OverflowError):  # floats and the like: int() of each, its low 32 bits
+        return array.array("i", [ctypes.c_int32(int(x)).value for x in xs])
+
+
+def _doubles(xs):
+    try:
+        return array.array("d", xs)
+    except TypeError:
+        return array.array("d", [float(x) for x in xs])
 
 
 def _check(code, where):
@@ -123,13 +151,13 @@ def spec_allocate(conf, cand_T, cand_cost, last_tokens, draft_tokens, pos_base, 
     """conf [B, K] fp32 device; cand_T / cand_cost host sequences; see spec.h."""
     B, K = conf.shape
     M = len(cand_T)
-    T = (ctypes.c_int32 * M)(*[int(x) for x in cand_T])
-    C = (ctypes.c_double * M)(*[float(x) for x in cand_cost])
+    T = _int32s(cand_T)
+    C = _doubles(cand_cost)
     code = library().spec_allocate(
-        _ptr(conf), B, K, T, C, M, _ptr(last_tokens), _ptr(draft_tokens), _ptr(pos_base),
-        _ptr(depth_out), _ptr(row_offsets_out), _ptr(packed_tokens_out), _ptr(packed_pos_out),
-        _ptr(chosen_T_out), _ptr(utility_out), _ptr(status), _ptr(ws),
-        0 if ws is None else ws.numel() * ws.element_size(), _stream(stream))
+        _ptr(conf), B, K, T.buffer_info()[0], C.buffer_info()[0], M, _ptr(last_tokens),
+        _ptr(draft_tokens), _ptr(pos_base), _ptr(depth_out), _ptr(row_offsets_out),
+        _ptr(packed_tokens_out), _ptr(packed_pos_out), _ptr(chosen_T_out), _ptr(utility_out),
+        _ptr(status), _ptr(ws), _nbytes(ws), _stream(stream))
     _check(code, "spec_allocate")
 
 
@@ -153,8 +181,7 @@ def spec_verify(logits, draft_tokens, q, B, K, V, temperature, seeds, request_id
         _ptr(logits), _dtype(logits), _ptr(row_offsets), _ptr(depth), _ptr(draft_tokens),
         _ptr(q), _dtype(q), B, K, V, float(temperature), _ptr(seeds), _ptr(request_ids),
         _ptr(pos_base), _ptr(accepted_len_out), _ptr(out_tokens), _ptr(p_draft_out),
-        _ptr(row_stats_out), _ptr(status), _ptr(ws), ws.numel() * ws.element_size(),
-        _stream(stream))
+        _ptr(row_stats_out), _ptr(status), _ptr(ws), ws.nbytes, _stream(stream))
     _check(code, "spec_verify")
 
 
@@ -282,7 +309,7 @@ def shard_workspace(B: int, K: int, V_shard: int, device="cuda"):
 
 
 def _nbytes(t):
-    return 0 if t is None else t.numel() * t.element_size()
+    return 0 if t is None else t.nbytes
 
 
 def spec_shard_stats(logits_shard, draft_tokens, q_shard, B, K, V, v_begin, temperature, pos_base,

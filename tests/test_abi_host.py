@@ -216,3 +216,38 @@ def test_pointer_readability_without_a_device(lib):
     assert lib.spec_pointer_device_readable(None) == 0
     buf = ctypes.create_string_buffer(64)
     assert lib.spec_pointer_device_readable(ctypes.cast(buf, ctypes.c_void_p)) in (0, 1)
+
+
+def test_candidate_lists_marshal_as_before():
+    """Budgets and costs from any host sequence reach the library as the int32
+    and double of each entry: lists, tuples, numpy arrays and scalars, torch
+    tensors, whole-valued floats."""
+    import numpy as np
+    import torch
+
+    import paper_2607_25852_gb300 as spec
+    want = [4, 272, 8192]
+    for xs in (want, tuple(want), np.asarray(want, np.int64), np.asarray(want, np.int32), [4.0, 272.9, 8192.0],
+               torch.tensor(want), [np.int64(4), np.int32(272), torch.tensor(8192)]):
+        assert list(spec._int32s(xs)) == want
+    assert list(spec._int32s([2**32 + 7, -(2**40) - 1])) == [7, -1]  # the low 32 bits, as ctypes takes them
+    for xs in ([1, 2.5], (np.float32(1), 2.5), np.asarray([1.0, 2.5]), torch.tensor([1.0, 2.5], dtype=torch.float64),
+               ["1", "2.5"]):
+        assert list(spec._doubles(xs)) == [1.0, 2.5]
+
+
+def test_pointer_arguments_keep_their_checks():
+    import pytest
+    import torch
+
+    import paper_2607_25852_gb300 as spec
+    assert spec._ptr(None) is None
+    t = torch.zeros(4, 6)
+    assert spec._ptr(t) == t.data_ptr()
+    with pytest.raises(ValueError):
+        spec._ptr(t.t())
+    with pytest.raises(TypeError):
+        spec._ptr([1, 2])
+    with pytest.raises(TypeError):
+        spec._dtype(t.double())
+    assert (spec._dtype(None), spec._dtype(t), spec._dtype(t.bfloat16())) == (spec.BF16, spec.F32, spec.BF16)
