@@ -39,25 +39,57 @@ namespace spec {
 static inline long long ceil_div(long long a, long long b) { return (a + b - 1) / b; }
 static inline long long round_up(long long a, long long b) { return ceil_div(a, b) * b; }
 
+// Streaming pass over R rows: the chunks per row with the least waves x (load
+// rounds of a chunk + 1), over waves of four CTAs on 152 SMs and rounds of 256
+// threads x 8 16-byte vectors (16384 bf16 entries); the 1 stands for a CTA's
+// start and its reduction.  Long chunks win because a CTA's rounds follow one
+// another without them, unless a second, mostly empty wave follows.  Measured
+// (us a call, replayed from a graph) against ~4096 CTAs whatever the shape:
+// B=64, K=16, V=65536, t=1: 31.1 (one chunk) / 37.9; V=201088: 78.3 / 80.3;
+// B=32: 44.4 / 47.6; B=32, K=8, V=151936 with dense q: 25.2 (two chunks) /
+// 27.1; B=16, K=16, V=128256, t=0: 12.7 (two) / 13.6.
+static void stream_chunks(long long R, long long V, int& nc_out, int& chunk_out) {
+  constexpr long long kRound = 16384, kSlots = 152 * 4;
+  long long nc = 1, best = LLONG_MAX;
+  const long long nc_max = std::max(1LL, std::min(V / kRound, ceil_div(2 * kSlots, R)));
+  for (long long n = 1; n <= nc_max; ++n) {
+    const long long cost = ceil_div(R * n, kSlots) * (ceil_div(ceil_div(V, n), kRound) + 1);
+    if (cost <= best) {  // a tie takes the shorter chunks
+      best = cost;
+      nc = n;
+    }
+  }
+  // whole rounds, so that only a row's last chunk ends in a partial one, where
+  // that keeps the number of chunks
+  long long chunk = round_up(ceil_div(V, nc), kRound);
+  if (ceil_div(V, chunk) < nc) chunk = round_up(ceil_div(V, nc), 2048);
+  nc_out = (int)ceil_div(V, chunk);  // every chunk non-empty
+  chunk_out = (int)chunk;
+}
+
 VerifyGeometry verify_geometry(int B, int K, int V) {
   VerifyGeometry g{};
   const long long R_max = (long long)B * (K + 1);
-  // Streaming pass: aim for ~4096 (row, chunk) items, each a whole number of
-  // load rounds (256 threads x 8 16-byte vectors = 16384 bf16 entries), so
-  // that only the last chunk of a row ends in a partial round.
-  long long nc = ceil_div(4096, R_max);
-  nc = std::max(1LL, std::min(nc, std::max(1LL, (long long)V / 16384)));
-  long long chunk = round_up(ceil_div(V, nc), 16384);
-  nc = ceil_div(V, chunk);  // every chunk non-empty
+  stream_chunks(R_max, V, g.NC, g.chunk);
+  // Packed rows: between B and R_max of them, known on the device only.  The
+  // chunks suit a quarter of the full block, D-cut's smallest budget; for more
+  // rows they are a little short (B=64, K=16, V=201088, all rows: 1 % slower
+  // than the line above), and one chunk per row leaves a quarter of the SMs'
+  // slots empty where few are kept (272 rows of V=128256: 10 % slower).
+  stream_chunks(std::max<long long>(B, R_max / 4), V, g.NC_packed, g.chunk_packed);
+  const long long nc = std::max(g.NC, g.NC_packed);
   // Sampling pass: aim for ~560 (request, chunk) CTAs, about one resident
   // wave on 152 SMs, of >= 2048 elements each, every chunk a whole number of
   // race quads (1024 entries).
   long long ncs = ceil_div(560, B);
   ncs = std::max(1LL, std::min(ncs, std::max(1LL, (long long)V / 2048)));
   long long chunk_s = round_up(ceil_div(V, ncs), 1024);
+  // A CTA's eight warps take a quad each at a time: whole rounds of eight
+  // quads, if the CTAs still fit one wave of four per SM (B=32, V=151936, dense
+  // q: 28.5 us a call with eight quads a CTA, 29.5 with nine).
+  const long long even = chunk_s / 8192 * 8192;
+  if (even > 0 && ceil_div(V, even) * B <= 608) chunk_s = even;
   ncs = ceil_div(V, chunk_s);
-  g.NC = (int)nc;
-  g.chunk = (int)chunk;
   g.NCS = (int)ncs;
   g.chunk_s = (int)chunk_s;
   g.row_part_off = 0;
@@ -195,11 +227,35 @@ __device__ __forceinline__ StreamItem stream_item(const VerifyLaunch& p) {
   return it;
 }
 
+// Before the grid-dependency wait, while the previous kernel on the stream
+// (the allocator, say: one CTA, HBM idle) drains: a line a thread of the
+// logits towards L2.  A prefetch returns no data, and L2 is where the previous
+// kernel's writes arrive, so nothing is read early.  Without row offsets it is
+// the CTA's own first load round; with them the row is not known yet, and the
+// CTAs in order take rows 0 .. B-1, which every packing holds.  Measured a call:
+// B=16, K=16, V=128256, t=0: 13.5 us with, 15.9 without; B=32, K=8, V=151936,
+// dense q: 27.0 / 28.4; the stress round (allocate, verify, commit): 92.2 / 93.8.
+template <typename T>
+__device__ __forceinline__ void prefetch_first_round(const VerifyLaunch& p, const StreamItem& it) {
+  constexpr int kLine = 128 / (int)sizeof(T);
+  long long v, end;
+  if (p.row_offsets) {
+    v = ((long long)blockIdx.x * kStreamThreads + threadIdx.x) * kLine;
+    end = (long long)p.B * p.V;
+  } else {
+    const long long row = ((long long)it.i * (p.K + 1) + it.j) * p.V;
+    v = row + (long long)it.c * p.chunk + (long long)threadIdx.x * kLine;
+    end = row + min((long long)p.V, (long long)(it.c + 1) * p.chunk);
+  }
+  if (v < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const T*>(p.logits) + v));
+}
+
 // Streaming pass with 16-byte loads from global memory (any alignment: a
 // scalar head and tail around the aligned body).
 template <typename T, bool kGreedy>
 __global__ void __launch_bounds__(kStreamThreads, kGreedy ? 4 : 0) stream_rows_kernel(const VerifyLaunch p) {
   const StreamItem it = stream_item(p);
+  prefetch_first_round<T>(p, it);
   pdl_wait_prerequisites();  // row offsets and depths come from the allocator
   const ReqShape rs = request_shape(p, it.i);
   if (!(rs.valid ? it.j <= rs.n : (it.j == 0 && it.c == 0))) return;

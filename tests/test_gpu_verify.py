@@ -210,3 +210,19 @@ def test_misaligned_logits_and_q(t):
     ref = run_oracle(wl.logits, wl.drafts, wl.q, t, wl.seeds, wl.request_ids, wl.pos_base)
     assert gpu["status"] == 0 and (ref["status"] == 0).all()
     compare(gpu, ref, wl.K, t)
+
+
+# Chunks per row by shape: one to six, of whole load rounds or (where that would
+# lose a chunk) of 2048 entries, the last one short; the same rows packed by an
+# allocation take their own chunks.  Sampling chunks of whole and of partial
+# rounds of eight quads.
+@pytest.mark.parametrize("B,K,V,dtype", [(1, 1, 40961, "bf16"), (2, 3, 65544, "bf16"), (12, 7, 100003, "f32"),
+                                         (3, 16, 151936, "bf16"), (8, 15, 70000, "bf16"), (40, 16, 33000, "bf16")])
+@pytest.mark.parametrize("t", [0.0, 0.8])
+def test_chunked_rows(B, K, V, dtype, t):
+    wl = _random_case(V, dtype, t, "dense" if t > 0 else "onehot", B=B, K=K, seed=B)
+    _check(wl, t)
+    depth = torch.as_tensor(np.random.default_rng(B).integers(0, K + 1, B), dtype=torch.int32)
+    offs = torch.cat([torch.zeros(1, dtype=torch.int32), torch.cumsum(depth + 1, 0).to(torch.int32)])
+    packed = workloads.pack_rows(wl.logits, B, K, depth)
+    _check(wl, t, depth=depth, row_offsets=offs, logits=packed)
