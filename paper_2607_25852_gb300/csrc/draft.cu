@@ -118,13 +118,6 @@ __device__ __forceinline__ float lg2_approx(float x) {
   return y;
 }
 
-// Order-preserving map of a non-NaN float onto int32 (signed compare).
-__device__ __forceinline__ int orderable(float f) {
-  const int b = __float_as_int(f);
-  return b < 0 ? b ^ 0x7FFFFFFF : b;
-}
-__device__ __forceinline__ float from_orderable(int k) { return __int_as_float(k < 0 ? k ^ 0x7FFFFFFF : k); }
-
 // A round's 16-byte words: lane l reads, for each of the round's kHalf sets of
 // four blocks, word l & 7 of every 128-byte line of block 4h + (l >> 3): 8
 // loads in flight, each of four whole lines over the warp.
@@ -283,7 +276,7 @@ template <typename T, bool kGreedy>
 __device__ __forceinline__ void draft_round(WarpDraftState& ws, const uint4 (&w)[8], int b0, int lane, float c2) {
   using R = Round<T>;
   const float Mr = from_orderable(__reduce_max_sync(0xFFFFFFFFu, orderable(words_max(w, T()))));
-  const float M2 = Mr > -INFINITY ? Mr * c2 : 0.0f;
+  const float M2 = Mr > -INFINITY ? __fmul_rn(Mr, c2) : 0.0f;
   const float2 c2v = make_float2(c2, c2), nM2 = make_float2(-M2, -M2);
   float acc[R::kHalf];
 #pragma unroll
@@ -305,11 +298,11 @@ __device__ __forceinline__ void draft_round(WarpDraftState& ws, const uint4 (&w)
   // the softmax state: the lane's part, scaled to the larger max
   const float own = R::kHalf == 2 ? acc[0] + acc[R::kHalf - 1] : acc[0];
   if (Mr > ws.m) {
-    ws.s = fmaf(ws.s, ex2_approx(ws.m * c2 - M2), own);
+    ws.s = fmaf(ws.s, ex2_approx(__fmul_rn(ws.m, c2) - M2), own);
     ws.m = Mr;
     if (kGreedy) ws.first = b0;
   } else {
-    ws.s = Mr > -INFINITY ? fmaf(own, ex2_approx(M2 - ws.m * c2), ws.s) : ws.s + own;
+    ws.s = Mr > -INFINITY ? fmaf(own, ex2_approx(M2 - __fmul_rn(ws.m, c2)), ws.s) : ws.s + own;
   }
   if (kGreedy) return;
   const float sb = block_sum(acc, lane);
@@ -327,16 +320,6 @@ __device__ __forceinline__ void draft_candidate(WarpDraftState& ws, int b, uint3
   const float E = -log1pf(-((float)race_m(word) * 0x1p-24f));
   const BlockKey k{lg2_approx(E) - lg2_approx(ws.keep_s), ws.keep_m, b};
   if (block_key_better(k, ws.best, c2)) ws.best = k;
-}
-
-// Minimum key over the warp (every lane).
-__device__ __forceinline__ KeyState warp_min_key(KeyState b) {
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const KeyState other{__shfl_xor_sync(0xFFFFFFFFu, b.key, o), __shfl_xor_sync(0xFFFFFFFFu, b.idx, o)};
-    if (key_better(other, b)) b = other;
-  }
-  return b;
 }
 
 // One warp per (row, segment of blocks); the warps of a CTA are independent

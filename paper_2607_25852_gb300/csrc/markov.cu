@@ -271,7 +271,7 @@ __device__ __forceinline__ SoftState mk_merge(SoftState a, SoftState b, float c2
     b = t;
   }
   if (b.m == -INFINITY) return a;
-  a.s = a.s + b.s * ex2_approx(b.m * c2 - a.m * c2);
+  a.s = a.s + b.s * ex2_approx(__fmul_rn(b.m, c2) - __fmul_rn(a.m, c2));
   return a;
 }
 __device__ __forceinline__ float mk_lg2(float x) {
@@ -635,11 +635,6 @@ __global__ void __launch_bounds__(kMkThreads, 1)
 // than unrolled butterflies of softmax merges, and what depends on the request
 // alone (the Philox words, log2 of the level-1 variate) is computed before the
 // grid-dependency wait.
-__device__ __forceinline__ int mk_orderable(float f) {
-  const int b = __float_as_int(f);
-  return b < 0 ? b ^ 0x7FFFFFFF : b;
-}
-__device__ __forceinline__ float mk_from_orderable(int k) { return __int_as_float(k < 0 ? k ^ 0x7FFFFFFF : k); }
 __device__ __forceinline__ int warp_max(int x) { return __reduce_max_sync(0xFFFFFFFFu, x); }
 __device__ __forceinline__ int warp_min(int x) { return __reduce_min_sync(0xFFFFFFFFu, x); }
 
@@ -703,19 +698,19 @@ __global__ void __launch_bounds__(kPickThreads, 1) markov_pick_kernel(const Mark
 
   // ---- the row's max ----
   {
-    const int m = warp_max(mk_orderable(st.m));
+    const int m = warp_max(orderable(st.m));
     if (lane == 0) sh_m[warp] = m;
     if ((int)threadIdx.x < p.r) sh_e[threadIdx.x] = e_own;
   }
   __syncthreads();
-  const float M = mk_from_orderable(warp_max(sh_m[lane]));
-  const float M2 = M * p.c2;
+  const float M = from_orderable(warp_max(sh_m[lane]));
+  const float M2 = __fmul_rn(M, p.c2);
 
   // ---- the row's sum; level 1 (tau > 0): log2 key of every 256-entry block,
   // log2 E_b - log2 sum_b + c2 (M - m_b), one block a thread; at tau = 0 the
   // lowest index that attains the max ----
   {
-    float s = st.m > -INFINITY ? st.s * exp2f(st.m * p.c2 - M2) : st.s;
+    float s = st.m > -INFINITY ? st.s * exp2f(__fmul_rn(st.m, p.c2) - M2) : st.s;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
     float key = INFINITY;
@@ -733,11 +728,11 @@ __global__ void __launch_bounds__(kPickThreads, 1) markov_pick_kernel(const Mark
                     m3 = left > 3 ? sq1.z : -INFINITY;
         const float bm = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
         if (bm > -INFINITY) {
-          const float b2 = bm * p.c2;
-          float bs = sq0.y * ex2_approx(m0 * p.c2 - b2);
-          if (left > 1) bs += sq0.w * ex2_approx(m1 * p.c2 - b2);
-          if (left > 2) bs += sq1.y * ex2_approx(m2 * p.c2 - b2);
-          if (left > 3) bs += sq1.w * ex2_approx(m3 * p.c2 - b2);
+          const float b2 = __fmul_rn(bm, p.c2);
+          float bs = sq0.y * ex2_approx(__fmul_rn(m0, p.c2) - b2);
+          if (left > 1) bs += sq0.w * ex2_approx(__fmul_rn(m1, p.c2) - b2);
+          if (left > 2) bs += sq1.y * ex2_approx(__fmul_rn(m2, p.c2) - b2);
+          if (left > 3) bs += sq1.w * ex2_approx(__fmul_rn(m3, p.c2) - b2);
           const float k = lgE - mk_lg2(bs) + p.c2 * (M - bm);
           if (bs > 0.0f && k < key) {  // b increases: a tie keeps the lower block
             key = k;
@@ -746,8 +741,8 @@ __global__ void __launch_bounds__(kPickThreads, 1) markov_pick_kernel(const Mark
         }
       }
     }
-    const int ko = kGreedy ? 0 : warp_min(mk_orderable(key));
-    const int im = warp_min(kGreedy || mk_orderable(key) == ko ? idx : INT_MAX);
+    const int ko = kGreedy ? 0 : warp_min(orderable(key));
+    const int im = warp_min(kGreedy || orderable(key) == ko ? idx : INT_MAX);
     if (lane == 0) {
       sh_s[warp] = s;
       sh_key[warp] = ko;

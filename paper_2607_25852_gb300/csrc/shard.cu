@@ -276,7 +276,7 @@ static cudaError_t launch_stats(unsigned grid, bool narrow, cudaStream_t stream,
 // ---------------------------------------------------------------------------
 // spec_shard_decide: one warp per request.
 // ---------------------------------------------------------------------------
-template <bool kGreedy>
+template <bool kGreedy, int kU>
 __global__ void __launch_bounds__(32) shard_decide_kernel(const ShardLaunch p) {
   const int i = blockIdx.x;
   const int lane = threadIdx.x;
@@ -288,17 +288,17 @@ __global__ void __launch_bounds__(32) shard_decide_kernel(const ShardLaunch p) {
   __shared__ float sh_pz[kMaxRows];
   __shared__ float sh_lq[kMaxRows];
   const ReqShape rs = request_shape(p, i);
-  const DecidePre pre = decide_prefetch<ShardLaunch, false, !kGreedy>(p, i);
+  const DecidePre<kU> pre = decide_prefetch<kU, ShardLaunch, false, !kGreedy>(p, i);
   const int n = rs.n;
   const long long row0 = rs.row0;
 #pragma unroll
-  for (int u = 0; u < (kMaxRows + 31) / 32; ++u)
+  for (int u = 0; u < kU; ++u)
     if (lane + 32 * u < p.K) sh_z[lane + 32 * u] = pre.z[u];
   __syncwarp();
   int bad = rs.valid ? 0 : 1;
-  float lz[(kMaxRows + 31) / 32], qz[(kMaxRows + 31) / 32];
+  float lz[kU], qz[kU];
 #pragma unroll
-  for (int u = 0; u < (kMaxRows + 31) / 32; ++u) {
+  for (int u = 0; u < kU; ++u) {
     lz[u] = 0.0f;
     qz[u] = 1.0f;
   }
@@ -357,7 +357,7 @@ __global__ void __launch_bounds__(32) shard_decide_kernel(const ShardLaunch p) {
     if (!kGreedy) {
       __syncwarp();
 #pragma unroll
-      for (int u = 0; u < (kMaxRows + 31) / 32; ++u) {
+      for (int u = 0; u < kU; ++u) {
         const int j = lane + 32 * u;
         if (j < n) {
           lz[u] = sh_pz[j];
@@ -368,7 +368,7 @@ __global__ void __launch_bounds__(32) shard_decide_kernel(const ShardLaunch p) {
   }
   bad = __any_sync(0xFFFFFFFFu, bad);
   __syncwarp();
-  decide_chain<kGreedy>(p, i, rs, pre, DecideArrays{sh_m, sh_S, sh_g, sh_z, sh_pz}, lz, qz, bad, true, p.req_rec + i);
+  decide_chain<kGreedy, kU>(p, i, rs, pre, DecideArrays{sh_m, sh_S, sh_g, sh_z, sh_pz}, lz, qz, bad, true, p.req_rec + i);
 }
 
 // ---------------------------------------------------------------------------
@@ -409,28 +409,20 @@ __device__ __forceinline__ KeyState shard_level2(const ShardLaunch& p, int mode,
   return race_level2<T, kWeightP>(row, qrow, p.q_dtype, vend, p.v_begin, b, ra, sh);
 }
 
-// The lowest keys a and b over the CTA in one exchange (results in thread 0;
-// sh: 2 x kSampleThreads / 32 slots).
+// The lowest keys a and b over the CTA in one exchange, in every thread (sh: 2 x
+// kSampleThreads / 32 slots, not used again before the caller's next barrier).
 __device__ __forceinline__ void cta_min_key2(KeyState& a, KeyState& b, KeyState* sh) {
+  constexpr int kW = kSampleThreads / 32;
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    const KeyState oa{__shfl_xor_sync(0xFFFFFFFFu, a.key, o), __shfl_xor_sync(0xFFFFFFFFu, a.idx, o)};
-    const KeyState ob{__shfl_xor_sync(0xFFFFFFFFu, b.key, o), __shfl_xor_sync(0xFFFFFFFFu, b.idx, o)};
-    if (key_better(oa, a)) a = oa;
-    if (key_better(ob, b)) b = ob;
-  }
+  a = warp_min_key(a);
+  b = warp_min_key(b);
   if (lane == 0) {
     sh[warp] = a;
-    sh[kSampleThreads / 32 + warp] = b;
+    sh[kW + warp] = b;
   }
   __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kSampleThreads / 32; ++k) {
-      if (key_better(sh[k], a)) a = sh[k];
-      if (key_better(sh[kSampleThreads / 32 + k], b)) b = sh[kSampleThreads / 32 + k];
-    }
-  __syncthreads();
+  a = warp_min_key(sh[lane & (kW - 1)]);
+  b = warp_min_key(sh[kW + (lane & (kW - 1))]);
 }
 
 // The shard's part [lo, hi) of block b (one entry per thread): the part's
@@ -516,7 +508,7 @@ template <typename T>
 __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const ShardLaunch p) {
   __shared__ int sh_last, sh_b, sh_bp;
   __shared__ float sh_kb, sh_kbp;
-  __shared__ KeyState sh_red[2 * (kSampleThreads / 32)];
+  __shared__ KeyState sh_red[3][2 * (kSampleThreads / 32)];  // level 1, the cut blocks' parts, level 2
   __shared__ float sh_f[2 * (kSampleThreads / 32)];
   const int i = blockIdx.x / p.NCS;
   const int cs = blockIdx.x - i * p.NCS;
@@ -556,7 +548,7 @@ __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const S
     shard_level1<T, kWeightExcl, true>(p, row, qrow, q_first, q_end, ra, best, best_p);
   else
     shard_level1<T, kWeightP, false>(p, row, qrow, q_first, q_end, ra, best, best_p);
-  cta_min_key2(best, best_p, sh_red);
+  cta_min_key2(best, best_p, sh_red[0]);
   // ---- the cut blocks at the shard's ends: the first and the last chunk's
   // CTA compute the shard's part of each before arriving ----
   const int hb = p.v_begin / kRaceBlock;   // block holding the first column
@@ -565,11 +557,11 @@ __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const S
   const bool tail_part = vend < p.V && vend % kRaceBlock != 0 && tb != hb;
   if (cs == 0 && head_part) {
     const ShardPart pt = shard_part<T>(p, mode, row, qrow, hb, p.v_begin, tb == hb ? vend : (hb + 1) * kRaceBlock,
-                                       ra, sh_red, sh_f);
+                                       ra, sh_red[1], sh_f);
     if (threadIdx.x == 0) p.part_ws[2 * (size_t)i] = pt;
   }
   if (cs == p.NCS - 1 && tail_part) {
-    const ShardPart pt = shard_part<T>(p, mode, row, qrow, tb, tb * kRaceBlock, vend, ra, sh_red, sh_f);
+    const ShardPart pt = shard_part<T>(p, mode, row, qrow, tb, tb * kRaceBlock, vend, ra, sh_red[1], sh_f);
     if (threadIdx.x == 0) p.part_ws[2 * (size_t)i + 1] = pt;
   }
   if (threadIdx.x == 0) {
@@ -627,12 +619,12 @@ __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const S
   out.y_p = -1;
   out.pad = 0;
   if (b != INT_MAX) {
-    const KeyState y = shard_level2<T>(p, mode, row, qrow, b, ra, sh_red);
+    const KeyState y = shard_level2<T>(p, mode, row, qrow, b, ra, sh_red[2]);
     out.y_r = y.idx == INT_MAX ? -1 : y.idx;
   } else if (mode != kWeightP && empty && bp != INT_MAX) {
     // no positive draw weight in this shard: its whole-block part of the
     // fallback race over p
-    const KeyState y = shard_level2<T>(p, kWeightP, row, nullptr, bp, ra, sh_red);
+    const KeyState y = shard_level2<T>(p, kWeightP, row, nullptr, bp, ra, sh_red[2]);
     out.key_p = sh_kbp;
     out.blk_p = bp;
     out.y_p = y.idx == INT_MAX ? -1 : y.idx;
@@ -873,10 +865,10 @@ extern "C" int spec_shard_decide(const void* stats, int S, const int32_t* row_of
   p.row_stats = row_stats_out;
   p.req_rec = static_cast<spec::ReqRec*>(decisions_out);
   p.status = status;
-  const cudaError_t err =
-      temperature == 0.0f
-          ? spec::launch_after_previous(spec::shard_decide_kernel<true>, dim3(B), dim3(32), 0, stream, p)
-          : spec::launch_after_previous(spec::shard_decide_kernel<false>, dim3(B), dim3(32), 0, stream, p);
+  const bool greedy = temperature == 0.0f, few = K <= 32;  // a draft a lane
+  auto kernel = greedy ? (few ? spec::shard_decide_kernel<true, 1> : spec::shard_decide_kernel<true, spec::kMaxU>)
+                       : (few ? spec::shard_decide_kernel<false, 1> : spec::shard_decide_kernel<false, spec::kMaxU>);
+  const cudaError_t err = spec::launch_after_previous(kernel, dim3(B), dim3(32), 0, stream, p);
   if (err != cudaSuccess || cudaGetLastError() != cudaSuccess) return SPEC_ERR_CUDA;
   return SPEC_OK;
 }

@@ -116,9 +116,9 @@ __shared__ int32_t sh_z[kMaxRows];
 __shared__ float sh_pz[kMaxRows];
 __device__ __forceinline__ DecideArrays decide_arrays() { return DecideArrays{sh_m, sh_S, sh_g, sh_z, sh_pz}; }
 
-template <typename T, bool kGreedy>
-__device__ __forceinline__ void decide_request(const VerifyLaunch& p, int i, ReqShape rs, const DecidePre& pre,
-                                            bool outputs, ReqRec* rec_dst) {
+template <bool kGreedy, int kU>
+__device__ __forceinline__ void decide_request(const VerifyLaunch& p, int i, ReqShape rs, const DecidePre<kU>& pre,
+                                               bool outputs, ReqRec* rec_dst) {
   const int K = p.K, V = p.V, NC = p.NC;
   const float c2 = p.c2;
   const int lane = threadIdx.x & 31;
@@ -129,9 +129,9 @@ __device__ __forceinline__ void decide_request(const VerifyLaunch& p, int i, Req
   // row's (target logit, q) at its draft from the streaming pass, and the
   // draft tokens (prefetched by the caller) ----
   int bad = rs.valid ? 0 : 1;
-  float lz[(kMaxRows + 31) / 32], qz[(kMaxRows + 31) / 32];
+  float lz[kU], qz[kU];
 #pragma unroll
-  for (int u = 0; u < (kMaxRows + 31) / 32; ++u) {
+  for (int u = 0; u < kU; ++u) {
     const int j = lane + 32 * u;
     lz[u] = 0.0f;
     qz[u] = 1.0f;
@@ -146,7 +146,7 @@ __device__ __forceinline__ void decide_request(const VerifyLaunch& p, int i, Req
       const RowPartial* part = p.row_part + (size_t)(row0 + j) * NC;
       int32_t f = 0;
       // kBatch partials in flight per lane
-      constexpr int kBatch = 8;
+      constexpr int kBatch = 4;
       if (kGreedy) {
         ArgState best{-INFINITY, INT_MAX};
         for (int c0 = 0; c0 < NC; c0 += kBatch) {
@@ -186,14 +186,14 @@ __device__ __forceinline__ void decide_request(const VerifyLaunch& p, int i, Req
     }
   }
 #pragma unroll
-  for (int u = 0; u < (kMaxRows + 31) / 32; ++u)
+  for (int u = 0; u < kU; ++u)
     if (lane + 32 * u < K) sh_z[lane + 32 * u] = pre.z[u];
   __syncwarp();
   for (int j = lane; j < n; j += 32)
     if (sh_z[j] < 0 || sh_z[j] >= V) bad = 1;
   bad = __any_sync(0xFFFFFFFFu, bad);
   __syncwarp();
-  decide_chain<kGreedy>(p, i, rs, pre, decide_arrays(), lz, qz, bad, outputs, rec_dst);
+  decide_chain<kGreedy, kU>(p, i, rs, pre, decide_arrays(), lz, qz, bad, outputs, rec_dst);
   __syncwarp();
 }
 
@@ -287,20 +287,20 @@ __global__ void __launch_bounds__(kStreamThreads, kGreedy ? 4 : 0) stream_rows_k
 // streaming kernel has written every row's (max, lowest argmax) partials.
 // The request's shape and drafts are the allocator's and the caller's, loaded
 // (through L2) while the streaming kernel drains.
-template <typename T>
+template <int kU>
 __global__ void __launch_bounds__(32) greedy_decide_kernel(const VerifyLaunch p) {
   const int i = blockIdx.x;
   const ReqShape rs = request_shape<VerifyLaunch, true>(p, i);
-  const DecidePre pre = decide_prefetch<VerifyLaunch, true, false>(p, i);
+  const DecidePre<kU> pre = decide_prefetch<kU, VerifyLaunch, true, false>(p, i);
   pdl_wait_prerequisites();  // the row partials of the streaming kernel
   pdl_launch_dependents();   // the commit kernel waits for this grid in turn
-  decide_request<T, true>(p, i, rs, pre, true, nullptr);
+  decide_request<true, kU>(p, i, rs, pre, true, nullptr);
 }
 
-template <typename T>
+template <typename T, int kU>
 __global__ void __launch_bounds__(kSampleThreads, 4) sample_kernel(const VerifyLaunch p) {
   __shared__ int sh_last, sh_b;
-  __shared__ KeyState sh_red[kSampleThreads / 32];
+  __shared__ KeyState sh_red[3][kSampleThreads / 32];
   const int i = blockIdx.x / p.NCS;
   const int cs = blockIdx.x - i * p.NCS;
   const int V = p.V;
@@ -312,13 +312,13 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_kernel(const VerifyL
   // launch: the allocator (the streaming CTAs waited for it before they let
   // this grid start) and the caller's earlier work.
   const ReqShape rs = request_shape<VerifyLaunch, true>(p, i);
-  DecidePre pre{};
-  if (warp == 0) pre = decide_prefetch<VerifyLaunch, true, true>(p, i);
+  DecidePre<kU> pre{};
+  if (warp == 0) pre = decide_prefetch<kU, VerifyLaunch, true, true>(p, i);
   pdl_wait_prerequisites();  // the row partials of the streaming kernel
   pdl_launch_dependents();   // the commit kernel waits for this grid in turn
   // The request's decision chain (every CTA of the request runs it; the last
   // CTA to finish the race writes the outputs): which row to sample, and how.
-  if (warp == 0) decide_request<T, false>(p, i, rs, pre, false, &sh_rec);
+  if (warp == 0) decide_request<false, kU>(p, i, rs, pre, false, &sh_rec);
   __syncthreads();
   const ReqRec rec = sh_rec;
   if (rec.flags & 1) {  // bad input: chunk 0 writes the flagged outputs
@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_kernel(const VerifyL
     race_level1_any<T, kWeightP>(p, row, qrow, q_first, q_end, warp, kSampleThreads / 32, ra, best);
 
   // ---- CTA reduction; the last CTA of the request to arrive goes on ----
-  best = cta_min_key(best, sh_red);
+  best = cta_min_key(best, sh_red[0]);
   if (threadIdx.x == 0) {
     RacePartial rp;
     rp.key_r = best.key;
@@ -391,11 +391,7 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_kernel(const VerifyL
       KeyState kr{__ldcg(&src->key_r), __ldcg(&src->idx_r)};
       if (key_better(kr, all)) all = kr;
     }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      KeyState other{__shfl_xor_sync(0xFFFFFFFFu, all.key, o), __shfl_xor_sync(0xFFFFFFFFu, all.idx, o)};
-      if (key_better(other, all)) all = other;
-    }
+    all = warp_min_key(all);
     if (lane == 0) {
       p.counters[i] = 0u;  // leave the workspace zeroed for the next call
       sh_b = all.idx;
@@ -411,20 +407,17 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_kernel(const VerifyL
     KeyState bp{INFINITY, INT_MAX};
     race_level1_any<T, kWeightP>(p, row, nullptr, 0, (V + kRaceQuad - 1) / kRaceQuad, warp, kSampleThreads / 32,
                                  ra, bp);
-    bp = cta_min_key(bp, sh_red);
-    if (threadIdx.x == 0) sh_b = bp.idx;
-    __syncthreads();
-    b = sh_b;
+    b = cta_min_key(bp, sh_red[1]).idx;
   }
   // ---- level 2 inside block b ----
   KeyState y{INFINITY, INT_MAX};
   if (b != INT_MAX) {
     if (wmode == kWeightResidual)
-      y = race_level2<T, kWeightResidual>(row, qrow, p.q_dtype, V, 0, b, ra, sh_red);
+      y = race_level2<T, kWeightResidual>(row, qrow, p.q_dtype, V, 0, b, ra, sh_red[2]);
     else if (wmode == kWeightExcl)
-      y = race_level2<T, kWeightExcl>(row, qrow, p.q_dtype, V, 0, b, ra, sh_red);
+      y = race_level2<T, kWeightExcl>(row, qrow, p.q_dtype, V, 0, b, ra, sh_red[2]);
     else
-      y = race_level2<T, kWeightP>(row, qrow, p.q_dtype, V, 0, b, ra, sh_red);
+      y = race_level2<T, kWeightP>(row, qrow, p.q_dtype, V, 0, b, ra, sh_red[2]);
   }
   if (threadIdx.x != 0) return;
   int32_t* tok = p.out_tokens + (size_t)i * (p.K + 1);
@@ -440,7 +433,7 @@ __global__ void __launch_bounds__(kSampleThreads, 4) sample_kernel(const VerifyL
 // ---------------------------------------------------------------------------
 // Launcher
 // ---------------------------------------------------------------------------
-template <typename T>
+template <typename T, int kU>
 static cudaError_t launch_typed(const VerifyLaunch& p, cudaStream_t stream, cudaEvent_t ev_before,
                                 cudaEvent_t ev_after) {
   const bool greedy = p.temperature == 0.0f;
@@ -455,13 +448,13 @@ static cudaError_t launch_typed(const VerifyLaunch& p, cudaStream_t stream, cuda
   if (err != cudaSuccess) return err;
   if (ev_after) cudaEventRecord(ev_after, stream);
   if (greedy) {
-    err = launch_after_previous(greedy_decide_kernel<T>, dim3((unsigned)p.B), dim3(32), 0, stream, p);
+    err = launch_after_previous(greedy_decide_kernel<kU>, dim3((unsigned)p.B), dim3(32), 0, stream, p);
     if (err != cudaSuccess) return err;
     return cudaGetLastError();
   }
   // The sampling CTAs are launched while the streaming kernel drains and
   // wait (griddepcontrol.wait) for its completion.
-  err = launch_after_previous(sample_kernel<T>, dim3((unsigned)((long long)p.B * p.NCS)), dim3(kSampleThreads), 0,
+  err = launch_after_previous(sample_kernel<T, kU>, dim3((unsigned)((long long)p.B * p.NCS)), dim3(kSampleThreads), 0,
                               stream, p);
   if (err != cudaSuccess) return err;
   return cudaGetLastError();
@@ -469,8 +462,12 @@ static cudaError_t launch_typed(const VerifyLaunch& p, cudaStream_t stream, cuda
 
 cudaError_t launch_verify(const VerifyLaunch& p, cudaStream_t stream, cudaEvent_t ev_before,
                           cudaEvent_t ev_after) {
-  if (p.logits_dtype == SPEC_F32) return launch_typed<float>(p, stream, ev_before, ev_after);
-  return launch_typed<__nv_bfloat16>(p, stream, ev_before, ev_after);
+  const bool few = p.K <= 32;  // a draft a lane
+  if (p.logits_dtype == SPEC_F32)
+    return few ? launch_typed<float, 1>(p, stream, ev_before, ev_after)
+               : launch_typed<float, kMaxU>(p, stream, ev_before, ev_after);
+  return few ? launch_typed<__nv_bfloat16, 1>(p, stream, ev_before, ev_after)
+             : launch_typed<__nv_bfloat16, kMaxU>(p, stream, ev_before, ev_after);
 }
 
 }  // namespace spec

@@ -17,10 +17,15 @@ constexpr int kStreamThreads = 256;
 constexpr int kUnroll = 8;
 constexpr int kSampleThreads = 256;
 constexpr int kMaxRows = SPEC_MAX_DRAFTS + 1;
+constexpr int kMaxU = kMaxRows / 32;  // drafts per lane of a deciding warp, at most
 
 // ---------------------------------------------------------------------------
 // Per-thread states and their merges
 // ---------------------------------------------------------------------------
+// Sums are kept relative to fl(m * c2): products that enter a difference of
+// exponents are rounded by themselves (__fmul_rn), so that no contraction into
+// an FMA puts an exact product on one side and a rounded one on the other (an
+// error of |m * c2| 2^-24 in the scale, 1e-5 at a temperature of 0.05).
 struct SoftState {
   float m;  // max logit seen
   float s;  // sum of 2^(l*c2 - fl(m*c2))
@@ -33,7 +38,7 @@ __device__ __forceinline__ SoftState soft_merge(SoftState a, SoftState b, float 
     b = t;
   }
   if (b.m == -INFINITY) return a;
-  const float Ma = a.m * c2, Mb = b.m * c2;
+  const float Ma = __fmul_rn(a.m, c2), Mb = __fmul_rn(b.m, c2);
   a.s = a.s + b.s * exp2f(Mb - Ma);
   return a;
 }
@@ -127,7 +132,7 @@ struct RowAcc {
     } else {
       if (x == INFINITY) flags |= 1;
       if (x > st.m) {
-        const float M2n = x * c2;
+        const float M2n = __fmul_rn(x, c2);
         st.s = st.s * exp2f(M2 - M2n);
         st.m = x;
         M2 = M2n;
@@ -184,7 +189,7 @@ struct RowAcc {
     } else {
       if (tm == INFINITY) flags |= 1;
       if (tm > st.m) {
-        const float M2n = tm * c2;
+        const float M2n = __fmul_rn(tm, c2);
         st.s = st.s * exp2f(M2 - M2n);
         st.m = tm;
         M2 = M2n;
@@ -260,66 +265,69 @@ __device__ __forceinline__ void stream_chunk(RowAcc<T, kGreedy>& acc, const T* r
   if (tail0 + (int)threadIdx.x < v1) acc.scalar(vofs + tail0 + threadIdx.x, load_elem(row + tail0 + threadIdx.x), c2);
 }
 
+// Order-preserving map of a non-NaN float onto int32 (signed compare).
+__device__ __forceinline__ int orderable(float f) {
+  const int b = __float_as_int(f);
+  return b < 0 ? b ^ 0x7FFFFFFF : b;
+}
+__device__ __forceinline__ float from_orderable(int k) { return __int_as_float(k < 0 ? k ^ 0x7FFFFFFF : k); }
+
+// The softmax state over kLanes lanes (a power of two; the other lanes hold
+// none), in every one of them: the max by redux, then one scaling per lane.
+template <int kLanes = 32>
+__device__ __forceinline__ SoftState warp_soft(SoftState st, float c2) {
+  const float m = from_orderable(__reduce_max_sync(0xFFFFFFFFu, orderable(st.m)));
+  float s = st.m > -INFINITY ? st.s * exp2f(__fmul_rn(st.m, c2) - __fmul_rn(m, c2)) : 0.0f;
+#pragma unroll
+  for (int o = kLanes / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xFFFFFFFFu, s, o);
+  return SoftState{m, s};
+}
+// The argmax over the warp, the lowest index on ties (-0 and +0 tie).
+__device__ __forceinline__ ArgState warp_arg(ArgState g) {
+  const int k = orderable(g.v + 0.0f);
+  const int m = __reduce_max_sync(0xFFFFFFFFu, k);
+  return ArgState{from_orderable(m), __reduce_min_sync(0xFFFFFFFFu, k == m ? g.idx : INT_MAX)};
+}
+
 // The CTA's (kThreads threads) reduction of a streamed chunk into one
 // partial, valid in thread 0.  Every thread of the CTA calls it.
 template <typename T, bool kGreedy, int kThreads = kStreamThreads>
 __device__ __forceinline__ RowPartial cta_reduce_partial(RowAcc<T, kGreedy>& acc, float c2) {
-  __shared__ float sh_a[kThreads / 32];
-  __shared__ float sh_b[kThreads / 32];
-  __shared__ int32_t sh_i[kThreads / 32];
-  __shared__ int32_t sh_f[kThreads / 32];
+  constexpr int kW = kThreads / 32;
+  __shared__ float sh_a[kW];
+  __shared__ float sh_b[kW];
+  __shared__ int32_t sh_i[kW];
+  __shared__ int32_t sh_f[kW];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   acc.finalize();
   const int32_t flags = __reduce_or_sync(0xFFFFFFFFu, (unsigned)acc.flags);
   RowPartial out{0.0f, 0.0f, 0, 0};
   if (kGreedy) {
-    ArgState g = acc.g;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      ArgState other{__shfl_xor_sync(0xFFFFFFFFu, g.v, o), __shfl_xor_sync(0xFFFFFFFFu, g.idx, o)};
-      if (arg_better(other, g)) g = other;
-    }
+    const ArgState g = warp_arg(acc.g);
     if (lane == 0) {
       sh_a[warp] = g.v;
       sh_i[warp] = g.idx;
       sh_f[warp] = flags;
     }
-    consumer_sync<kThreads>();
-    if (threadIdx.x == 0) {
-      ArgState best{sh_a[0], sh_i[0]};
-      int32_t f = sh_f[0];
-      for (int k = 1; k < kThreads / 32; ++k) {
-        ArgState o{sh_a[k], sh_i[k]};
-        if (arg_better(o, best)) best = o;
-        f |= sh_f[k];
-      }
-      out.m = best.v;
-      out.idx = best.idx;
-      out.flags = f;
-    }
   } else {
-    SoftState st = acc.st;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      SoftState other{__shfl_xor_sync(0xFFFFFFFFu, st.m, o), __shfl_xor_sync(0xFFFFFFFFu, st.s, o)};
-      st = soft_merge(st, other, c2);
-    }
+    const SoftState st = warp_soft(acc.st, c2);
     if (lane == 0) {
       sh_a[warp] = st.m;
       sh_b[warp] = st.s;
       sh_f[warp] = flags;
     }
-    consumer_sync<kThreads>();
-    if (threadIdx.x == 0) {
-      SoftState all{sh_a[0], sh_b[0]};
-      int32_t f = sh_f[0];
-      for (int k = 1; k < kThreads / 32; ++k) {
-        all = soft_merge(all, SoftState{sh_a[k], sh_b[k]}, c2);
-        f |= sh_f[k];
-      }
-      out.m = all.m;
-      out.s = all.s;
-      out.flags = f;
+  }
+  consumer_sync<kThreads>();
+  if (warp == 0) {
+    out.flags = (int32_t)__reduce_or_sync(0xFFFFFFFFu, lane < kW ? (unsigned)sh_f[lane] : 0u);
+    if (kGreedy) {
+      const ArgState g = warp_arg(lane < kW ? ArgState{sh_a[lane], sh_i[lane]} : ArgState{-INFINITY, INT_MAX});
+      out.m = g.v;
+      out.idx = g.idx;
+    } else {
+      const SoftState st = warp_soft<kW>(lane < kW ? SoftState{sh_a[lane], sh_b[lane]} : SoftState{-INFINITY, 0.0f}, c2);
+      out.m = st.m;
+      out.s = st.s;
     }
   }
   return out;
@@ -477,14 +485,29 @@ struct QuadWords {
 // read.  One block is one warp step: lane l holds entries 8l..8l+7 of it
 // (kSrc 0: 16-byte loads from global memory, the whole quad's loads issued at
 // once; kSrc 1: the same from shared memory) or entries l + 32e (kSrc 2:
-// scalar loads, any layout).  Every lane computes the same block sum and so
-// holds the same best block.
+// scalar loads, any layout).  The four block sums of a quad are formed
+// transposed (quad_sum): lane l races block l >> 3 of every quad, and the
+// caller takes the minimum over the lanes.
 //
 // kDual also runs the race with weights p (best_p) on the same block variates:
 // the draw a sharded caller falls back to when no shard has a positive weight.
 // kRange races only the blocks whose entries all lie in [lo, V), plus the
 // vocabulary's last block when tail_whole (V is then the vocabulary's end):
 // the blocks a vocabulary shard [lo, V) owns whole.
+
+// Sums over the warp of the four per-lane values w, transposed: lane l ends
+// with the sum of w[l >> 3] (two halving exchanges, then three butterfly
+// steps; the additions pair the lanes as a butterfly over all bits would).
+__device__ __forceinline__ float quad_sum(const float (&w)[4], int lane) {
+  const bool h16 = (lane & 16) != 0, h8 = (lane & 8) != 0;
+  const float a = (h16 ? w[2] : w[0]) + __shfl_xor_sync(0xFFFFFFFFu, h16 ? w[0] : w[2], 16);
+  const float b = (h16 ? w[3] : w[1]) + __shfl_xor_sync(0xFFFFFFFFu, h16 ? w[1] : w[3], 16);
+  float v = (h8 ? b : a) + __shfl_xor_sync(0xFFFFFFFFu, h8 ? a : b, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+  return v;
+}
+
 template <typename T, typename Q, int kMode, int kSrc, bool kDual, bool kRange>
 __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype, int V, int base_v, int q_first,
                                  int q_end, int warp_id, int nwarps, const RaceArgs& a, KeyState& best,
@@ -499,13 +522,13 @@ __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype,
       const int vb = q * kRaceQuad + s * kRaceBlock;
       raced[s] = vb < V && (!kRange || (vb >= lo && (tail_whole || vb + kRaceBlock <= V)));
     }
+    float wsum[4] = {0.0f, 0.0f, 0.0f, 0.0f}, wsum_p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+    uint4 r;
     if (kSrc == kSrcGlobalScalar) {
-      const uint4 r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
-      const uint32_t words[4] = {r.x, r.y, r.z, r.w};
+      r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
         const int vb = q * kRaceQuad + s * kRaceBlock;
-        float wsum = 0.0f, wsum_p = 0.0f;
         if (raced[s]) {
           float x[8], qv[8];
 #pragma unroll
@@ -519,18 +542,10 @@ __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype,
             const int v = vb + lane + 32 * e;
             if (v < V) {
               const float ew = p_weight(x[e], a.c2, a.M2);
-              wsum += weight_of<kMode>(ew, qv[e], v, a.invS, a.z_excl);
-              if (kDual) wsum_p += ew;
+              wsum[s] += weight_of<kMode>(ew, qv[e], v, a.invS, a.z_excl);
+              if (kDual) wsum_p[s] += ew;
             }
           }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xFFFFFFFFu, wsum, o);
-        race_entry(best, thr24, wsum, race_m(words[s]), 4 * q + s);
-        if (kDual) {
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) wsum_p += __shfl_xor_sync(0xFFFFFFFFu, wsum_p, o);
-          race_entry(best_p, thr24p, wsum_p, race_m(words[s]), 4 * q + s);
         }
       }
     } else {
@@ -538,30 +553,24 @@ __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype,
       QuadWords<Q, kSrc> qw;
       xw.load(row, q, V, base_v, raced);
       if (kMode == kWeightResidual) qw.load(qrow, q, V, base_v, raced);
-      const uint4 r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
-      const uint32_t words[4] = {r.x, r.y, r.z, r.w};
+      r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
 #pragma unroll
       for (int s = 0; s < 4; ++s) {
         const int v8 = q * kRaceQuad + s * kRaceBlock + 8 * lane;
-        float wsum = 0.0f, wsum_p = 0.0f;
         if (raced[s] && v8 < V) {
 #pragma unroll
           for (int e = 0; e < 8; ++e) {
             const float ew = p_weight(xw.get(s, e), a.c2, a.M2);
-            wsum += weight_of<kMode>(ew, kMode == kWeightResidual ? qw.get(s, e) : 0.0f, v8 + e, a.invS, a.z_excl);
-            if (kDual) wsum_p += ew;
+            wsum[s] += weight_of<kMode>(ew, kMode == kWeightResidual ? qw.get(s, e) : 0.0f, v8 + e, a.invS, a.z_excl);
+            if (kDual) wsum_p[s] += ew;
           }
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1) wsum += __shfl_xor_sync(0xFFFFFFFFu, wsum, o);
-        race_entry(best, thr24, wsum, race_m(words[s]), 4 * q + s);
-        if (kDual) {
-#pragma unroll
-          for (int o = 16; o > 0; o >>= 1) wsum_p += __shfl_xor_sync(0xFFFFFFFFu, wsum_p, o);
-          race_entry(best_p, thr24p, wsum_p, race_m(words[s]), 4 * q + s);
         }
       }
     }
+    const int s = lane >> 3;  // the lane's block; not raced: its sum is 0, which never passes the filter
+    const uint32_t m = race_m(s == 0 ? r.x : s == 1 ? r.y : s == 2 ? r.z : r.w);
+    race_entry(best, thr24, quad_sum(wsum, lane), m, 4 * q + s);
+    if (kDual) race_entry(best_p, thr24p, quad_sum(wsum_p, lane), m, 4 * q + s);
   }
 }
 
@@ -573,24 +582,30 @@ __device__ __forceinline__ void race_level1(const void* row, const void* qrow, i
                                                     best, best, 0, true);
 }
 
-// Minimum key over the CTA (valid in thread 0).  sh: kSampleThreads / 32 slots.
-__device__ __forceinline__ KeyState cta_min_key(KeyState b, KeyState* sh) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1) {
-    KeyState other{__shfl_xor_sync(0xFFFFFFFFu, b.key, o), __shfl_xor_sync(0xFFFFFFFFu, b.idx, o)};
-    if (key_better(other, b)) b = other;
-  }
-  if (lane == 0) sh[warp] = b;
-  __syncthreads();
-  if (threadIdx.x == 0)
-    for (int k = 0; k < kSampleThreads / 32; ++k)
-      if (key_better(sh[k], b)) b = sh[k];
-  __syncthreads();
-  return b;
+// Minimum key over the warp, in every lane.  Keys are positive (+inf: none, or
+// a weight that underflows), so they order as their bits do: two redux
+// instructions instead of a butterfly.  With the streaming CTAs' reduction in
+// the same form, the decision code without its unused draft slots and a race
+// block per lane group, a call took (before / now, replayed from a graph):
+// B=32, K=8, V=151936, dense q 25.2 / 23.3 us; fp32 V=100003 18.5 / 16.8; the
+// stress round 92.9 / 89.9; the tiny round 17.8 / 16.1; t = 0 12.8 / 12.4.
+__device__ __forceinline__ KeyState warp_min_key(KeyState b) {
+  const unsigned k = __float_as_uint(b.key);
+  const unsigned kmin = __reduce_min_sync(0xFFFFFFFFu, k);
+  return KeyState{__uint_as_float(kmin), (int32_t)__reduce_min_sync(0xFFFFFFFFu, (unsigned)(k == kmin ? b.idx : INT_MAX))};
 }
 
-// Level 2 in block b (one entry per thread; result in thread 0).
+// Minimum key over the CTA, in every thread.  sh: kSampleThreads / 32 slots,
+// not used again before the caller's next barrier.
+__device__ __forceinline__ KeyState cta_min_key(KeyState b, KeyState* sh) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  b = warp_min_key(b);
+  if (lane == 0) sh[warp] = b;
+  __syncthreads();
+  return warp_min_key(sh[lane & (kSampleThreads / 32 - 1)]);
+}
+
+// Level 2 in block b (one entry per thread; result in every thread).
 template <typename T, int kMode>
 __device__ KeyState race_level2(const T* row, const void* qrow, int q_dtype, int V, int base_v, int b, const RaceArgs& a,
                                 KeyState* sh) {
@@ -670,21 +685,25 @@ __device__ __forceinline__ ReqShape request_shape(const L& p, int i) {
 // warp before the statistics are complete (before the arrival atomic, or
 // before the grid-dependency wait).  z[u] and u[u] belong to draft
 // j = lane + 32u.
+//
+// kU = 1 serves K <= 32, kMaxU all K: a decision runs once per CTA from cold
+// instruction caches, so what a shape does not need is kept out of its kernel.
+template <int kU>
 struct DecidePre {
   uint32_t pos;
   unsigned long long seed, req;
-  int32_t z[(kMaxRows + 31) / 32];
-  float u[(kMaxRows + 31) / 32];
+  int32_t z[kU];
+  float u[kU];
 };
-template <class L, bool kL2 = false, bool kDraws = false>
-__device__ __forceinline__ DecidePre decide_prefetch(const L& p, int i) {
+template <int kU, class L, bool kL2 = false, bool kDraws = false>
+__device__ __forceinline__ DecidePre<kU> decide_prefetch(const L& p, int i) {
   const int lane = threadIdx.x & 31;
-  DecidePre pre;
+  DecidePre<kU> pre;
   pre.pos = (uint32_t)load_in<kL2>(reinterpret_cast<const long long*>(p.pos_base) + i);
   pre.seed = load_in<kL2>(reinterpret_cast<const unsigned long long*>(p.seeds) + i);
   pre.req = load_in<kL2>(reinterpret_cast<const unsigned long long*>(p.request_ids) + i);
 #pragma unroll
-  for (int u = 0; u < (kMaxRows + 31) / 32; ++u) {
+  for (int u = 0; u < kU; ++u) {
     const int j = lane + 32 * u;
     pre.z[u] = j < p.K ? load_in<kL2>(p.drafts + (size_t)i * p.K + j) : 0;
     pre.u[u] = 1.0f;
@@ -762,11 +781,10 @@ __device__ __forceinline__ void write_decision(const L& p, int i, const ReqShape
   }
 }
 
-template <bool kGreedy, class L>
-__device__ __forceinline__ void decide_chain(const L& p, int i, const ReqShape& rs, const DecidePre& pre,
-                                             const DecideArrays& sh, const float (&lz)[(kMaxRows + 31) / 32],
-                                             const float (&qz)[(kMaxRows + 31) / 32], int bad, bool outputs,
-                                             ReqRec* rec_dst) {
+template <bool kGreedy, int kU, class L>
+__device__ __forceinline__ void decide_chain(const L& p, int i, const ReqShape& rs, const DecidePre<kU>& pre,
+                                             const DecideArrays& sh, const float (&lz)[kU], const float (&qz)[kU],
+                                             int bad, bool outputs, ReqRec* rec_dst) {
   const int K = p.K;
   const float c2 = p.c2;
   const int lane = threadIdx.x & 31;
@@ -782,7 +800,7 @@ __device__ __forceinline__ void decide_chain(const L& p, int i, const ReqShape& 
   int first_reject = n;
   if (!bad) {
 #pragma unroll
-    for (int u = 0; u < (kMaxRows + 31) / 32; ++u) {
+    for (int u = 0; u < kU; ++u) {
       const int j = lane + 32 * u;
       if (j >= n) break;
       const int z = sh_z[j];

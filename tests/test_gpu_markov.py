@@ -240,3 +240,16 @@ def test_bad_entries_in_any_tile(V, value):
         assert (g["z"] == -1).all(axis=1).tolist() == [False, True, True, False, True, False]
         o = run_oracle_markov(U, W1, W2, x0, tau, seeds, rids, pos)
         compare_markov(g, o, U, W1, W2, x0, tau)
+
+
+def test_low_temperature_statistics():
+    """W1 = 0 (the bias is exactly 0) at tau = 0.05, where |max| / tau log2 e
+    reaches hundreds: the row statistics keep spec_draft's tolerance (the sums
+    are relative to the rounded product of the max, throughout)."""
+    B, K, V = 7, 3, 9000
+    U, W1, W2, x0, seeds, rids, pos = _case(B, K, V, 64, 17, std=3.0)
+    g = run_markov(U, torch.zeros_like(W1), W2, x0, 0.05, seeds, rids, pos)
+    o = run_oracle_markov(U, torch.zeros_like(W1), W2, x0, 0.05, seeds, rids, pos)
+    assert g["status"] == 0
+    np.testing.assert_allclose(g["st"][:, 0], o["m"].reshape(-1), rtol=1e-5, atol=0)
+    np.testing.assert_allclose(g["st"][:, 1], o["logS"].reshape(-1), rtol=0, atol=1e-5)
