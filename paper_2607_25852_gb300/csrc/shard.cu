@@ -139,7 +139,9 @@ static ShardGeometry shard_geometry(int B, int K, int Vs) {
   const long long chunk = ((Vs + nc - 1) / nc + 16383) / 16384 * 16384;
   s.NC = (int)((Vs + chunk - 1) / chunk);  // every chunk non-empty
   s.chunk = (int)chunk;
-  s.quads_s = g.chunk_s / kRaceQuad;
+  // at least a quad for each of a CTA's eight warps: a rank's round of 25136
+  // columns takes 31.5 us so, 32.1 us with three quads a CTA
+  s.quads_s = std::max(kSampleThreads / 32, g.chunk_s / kRaceQuad);
   // a shard of Vs columns spans at most ceil(Vs / 1024) + 1 quads
   const long long nq_max = (Vs + kRaceQuad - 1) / kRaceQuad + 1;
   s.NCS_max = (int)((nq_max + s.quads_s - 1) / s.quads_s);
@@ -323,6 +325,20 @@ __global__ void __launch_bounds__(32) shard_decide_kernel(const ShardLaunch p) {
             if (j < n) b[u] = rec[k + 1];
           }
         }
+        if (!kGreedy) {
+          // the batch's sums at its largest max: scalings that do not wait for
+          // one another, added in shard order
+          float m = all.m;
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u)
+            if (s0 + u < p.S) m = fmaxf(m, __uint_as_float(a[u].x));
+          const float M2 = m > -INFINITY ? __fmul_rn(m, p.c2) : 0.0f;
+          float s = all.m > -INFINITY ? all.s * exp2f(__fmul_rn(all.m, p.c2) - M2) : 0.0f;
+#pragma unroll
+          for (int u = 0; u < kBatch; ++u)
+            if (s0 + u < p.S) s += __uint_as_float(a[u].y) * exp2f(__fmul_rn(__uint_as_float(a[u].x), p.c2) - M2);
+          all = SoftState{m, s};
+        }
 #pragma unroll
         for (int u = 0; u < kBatch; ++u) {
           if (s0 + u >= p.S) break;
@@ -330,8 +346,6 @@ __global__ void __launch_bounds__(32) shard_decide_kernel(const ShardLaunch p) {
           if (kGreedy) {
             const ArgState o{__uint_as_float(a[u].x), (int32_t)a[u].z};
             if (arg_better(o, best)) best = o;
-          } else {
-            all = soft_merge(all, SoftState{__uint_as_float(a[u].x), __uint_as_float(a[u].y)}, p.c2);
           }
           if (j < n && b[u].z) {
             ++owners;
@@ -643,30 +657,42 @@ __device__ __forceinline__ uint32_t block_word(int b, const RaceArgs& a) {
   return (b & 3) == 0 ? r.x : (b & 3) == 1 ? r.y : (b & 3) == 2 ? r.z : r.w;
 }
 
-// Candidate block b with weight sum W (summed over its parts) and race word
-// `word`: key E_b / W.
-__device__ __forceinline__ void finish_block(KeyState& best, int& y, int b, float W, int y_part, uint32_t word) {
-  if (!(W > 0.0f)) return;
-  const KeyState k{race_key(race_m(word), W), b};
-  if (key_better(k, best)) {
-    best = k;
-    y = y_part;
-  }
-}
-
-// One warp per request: the lanes load up to 32 shards' records at a time
-// into shared memory, lane 0 merges them in shard order.
+// One warp per request, a lane per shard record (more than 32 shards: in
+// turn).  A lane takes its record's whole-block keys and the cut blocks that
+// start in its shard: their parts, added in shard order, are its own part and
+// the head parts of the shards that follow.  The lowest keys are then taken
+// over the lanes.  A rank's round (B = 64, K = 16, V = 201088, S = 8, replayed
+// as a graph) took 34.9 us with the records merged one after another by one
+// lane, here and in the decision; 32.1 us with both in this form.
 constexpr int kFinishWarps = 4;
 
+// A race candidate and the entry drawn for it.
+struct FinishBest {
+  KeyState k{INFINITY, INT_MAX};
+  int y = -1;
+  __device__ __forceinline__ void take(float key, int blk, int y_new) {
+    const KeyState n{key, blk};
+    if (blk != INT_MAX && key_better(n, k)) {
+      k = n;
+      y = y_new;
+    }
+  }
+  // over the warp: the entry of the lane that holds the lowest key
+  __device__ __forceinline__ void over_warp() {
+    const KeyState m = warp_min_key(k);
+    const unsigned who = __ballot_sync(0xFFFFFFFFu, k.idx == m.idx && k.key == m.key);
+    y = __shfl_sync(0xFFFFFFFFu, y, __ffs(who) - 1);
+    k = m;
+  }
+};
+
 __global__ void __launch_bounds__(32 * kFinishWarps) shard_finish_kernel(const ShardLaunch p) {
-  __shared__ ShardRace sh_rec[kFinishWarps][32];
-  __shared__ uint32_t sh_word[kFinishWarps][32][2];  // the race words of the records' cut blocks
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int i = blockIdx.x * kFinishWarps + warp;
   pdl_wait_prerequisites();
   if (i >= p.B) return;
   const ReqRec rec = p.req_rec[i];
-  if (rec.flags & 1) return;
+  if (rec.flags & 1) return;  // bad input: the decision wrote the outputs
   if (rec.a < 0 || rec.a > p.K) {
     if (lane == 0) report(p.status, SPEC_ERR_WORKSPACE);
     return;
@@ -677,68 +703,42 @@ __global__ void __launch_bounds__(32 * kFinishWarps) shard_finish_kernel(const S
   const uint64_t seed = __ldg(reinterpret_cast<const unsigned long long*>(p.seeds) + i);
   a.k0 = (uint32_t)seed;
   a.k1 = (uint32_t)(seed >> 32);
-  KeyState r{INFINITY, INT_MAX}, q{INFINITY, INT_MAX};
-  int yr = -1, yq = -1;
-  // cut blocks: the parts of one block are adjacent in shard order
-  int cur = INT_MAX;
-  uint32_t cur_word = 0;
-  float Wr = 0.0f, Wp = 0.0f;
-  KeyState er{INFINITY, INT_MAX}, ep{INFINITY, INT_MAX};
-  for (int s0 = 0; s0 < p.S; s0 += 32) {
-    __syncwarp();
-    if (s0 + lane < p.S) {
-      const uint4* src = reinterpret_cast<const uint4*>(p.races + (size_t)(s0 + lane) * p.B + i);
-      uint4* dst = reinterpret_cast<uint4*>(&sh_rec[warp][lane]);
-#pragma unroll
-      for (int w = 0; w < (int)(sizeof(ShardRace) / 16); ++w) dst[w] = src[w];
-      // the race words of this record's cut blocks, a lane per record (lane
-      // 0 then merges the records in shard order)
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int b = sh_rec[warp][lane].part[h].blk;
-        sh_word[warp][lane][h] = b != INT_MAX ? block_word(b, a) : 0u;
-      }
+  FinishBest r, q;
+  for (int s = lane; s < p.S; s += 32) {
+    const ShardRace* x = p.races + (size_t)s * p.B + i;
+    const ShardRace own = *x;
+    // the block that the shard before ends in, if it is cut there
+    int before = INT_MAX;
+    if (s > 0) {
+      const ShardRace* prev = x - p.B;
+      before = prev->part[1].blk != INT_MAX ? prev->part[1].blk : prev->part[0].blk;
     }
-    __syncwarp();
-    if (lane != 0) continue;
-    for (int s = s0; s < min(p.S, s0 + 32); ++s) {
-      const ShardRace& x = sh_rec[warp][s - s0];
-      const KeyState kr{x.key_r, x.blk_r}, kp{x.key_p, x.blk_p};
-      if (x.blk_r != INT_MAX && key_better(kr, r)) {
-        r = kr;
-        yr = x.y_r;
+    r.take(own.key_r, own.blk_r, own.y_r);
+    q.take(own.key_p, own.blk_p, own.y_p);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+      const ShardPart& pt = own.part[h];
+      if (pt.blk == INT_MAX || (h == 0 && pt.blk == before)) continue;  // no such part, or the block starts earlier
+      float Wr = pt.w_r, Wp = pt.w_p;
+      KeyState er{pt.ek_r, pt.ey_r}, ep{pt.ek_p, pt.ey_p};
+      for (int t = s + 1; t < p.S; ++t) {  // the shards after it that hold a part of the block
+        const ShardPart nx = x[(size_t)(t - s) * p.B].part[0];
+        if (nx.blk != pt.blk) break;
+        Wr += nx.w_r;
+        Wp += nx.w_p;
+        const KeyState kr{nx.ek_r, nx.ey_r}, kp{nx.ek_p, nx.ey_p};
+        if (nx.ey_r != INT_MAX && key_better(kr, er)) er = kr;
+        if (nx.ey_p != INT_MAX && key_better(kp, ep)) ep = kp;
       }
-      if (x.blk_p != INT_MAX && key_better(kp, q)) {
-        q = kp;
-        yq = x.y_p;
-      }
-      for (int h = 0; h < 2; ++h) {
-        const ShardPart& pt = x.part[h];
-        if (pt.blk == INT_MAX) continue;
-        if (pt.blk != cur) {
-          if (cur != INT_MAX) {
-            finish_block(r, yr, cur, Wr, er.idx, cur_word);
-            finish_block(q, yq, cur, Wp, ep.idx, cur_word);
-          }
-          cur = pt.blk;
-          cur_word = sh_word[warp][s - s0][h];
-          Wr = Wp = 0.0f;
-          er = ep = KeyState{INFINITY, INT_MAX};
-        }
-        Wr += pt.w_r;
-        Wp += pt.w_p;
-        const KeyState kr2{pt.ek_r, pt.ey_r}, kp2{pt.ek_p, pt.ey_p};
-        if (pt.ey_r != INT_MAX && key_better(kr2, er)) er = kr2;
-        if (pt.ey_p != INT_MAX && key_better(kp2, ep)) ep = kp2;
-      }
+      const uint32_t m = race_m(block_word(pt.blk, a));
+      if (Wr > 0.0f) r.take(race_key(m, Wr), pt.blk, er.idx);
+      if (Wp > 0.0f) q.take(race_key(m, Wp), pt.blk, ep.idx);
     }
   }
+  r.over_warp();
+  q.over_warp();
   if (lane != 0) return;
-  if (cur != INT_MAX) {
-    finish_block(r, yr, cur, Wr, er.idx, cur_word);
-    finish_block(q, yq, cur, Wp, ep.idx, cur_word);
-  }
-  const int y = r.idx != INT_MAX ? yr : yq;
+  const int y = r.k.idx != INT_MAX ? r.y : q.y;
   int32_t* tok = p.out_tokens + (size_t)i * (p.K + 1);
   if (y < 0 || y >= p.V) {
     report(p.status, SPEC_ERR_BAD_INPUT);

@@ -237,3 +237,23 @@ def test_replay_and_workspace_reuse_are_bit_identical():
                     wl.pos_base, bounds, ws=a["ws"])
     for k in ("accepted", "tokens", "p_draft", "row_stats"):
         assert np.array_equal(a[k], b[k]) and np.array_equal(b[k], c[k]), k
+
+
+# The finish step's cut blocks: blocks over two, three and many shards, shards
+# inside one block, shards that end on a block boundary, more shards than the 32
+# lanes take at once; one-hot q (rejections exclude the draft) and dense q.
+@pytest.mark.parametrize("bounds", [
+    [0, 100, 200, 300, 1000],                        # a block over three shards, then one that starts cut
+    [0, 256, 512, 700, 1000],                        # whole blocks, then a cut
+    [0, 1, 2, 3, 255, 256, 257, 900, 1000],          # one-column shards at a block's ends
+    [25 * k for k in range(41)],                     # 40 shards, a dozen to a block
+    [0] + [7 * k + 3 for k in range(1, 142)] + [1000],  # 142 shards
+])
+@pytest.mark.parametrize("dense", [False, True])
+def test_cut_blocks(bounds, dense):
+    V = bounds[-1]
+    wl = _random_case(V, "f32", 0.9, "dense" if dense else "onehot", B=9, K=3, seed=len(bounds))
+    gpu = run_sharded(wl.logits, wl.drafts, wl.q, wl.B, wl.K, V, 0.9, wl.seeds, wl.request_ids, wl.pos_base, bounds)
+    ref = run_oracle(wl.logits, wl.drafts, wl.q, 0.9, wl.seeds, wl.request_ids, wl.pos_base)
+    assert gpu["status"] == 0 and (ref["status"] == 0).all()
+    compare(gpu, ref, wl.K, 0.9)
