@@ -512,20 +512,21 @@ __global__ void __launch_bounds__(kAllocThreads) allocate_small_kernel(const All
     uint32_t dst = (uint32_t)__cvta_generic_to_shared(&sh_x[1][0]);
     sts_u64(src + 8u * (uint32_t)tid, x);
     __syncthreads();
-    // the levels from runs of KP on, each unrolled for its L
-    switch (31 - __clz(KP)) {
-      case 0: merge_level<1>(x, tid, src, dst); [[fallthrough]];
-      case 1: merge_level<2>(x, tid, src, dst); [[fallthrough]];
-      case 2: merge_level<4>(x, tid, src, dst); [[fallthrough]];
-      case 3: merge_level<8>(x, tid, src, dst); [[fallthrough]];
-      case 4: merge_level<16>(x, tid, src, dst); [[fallthrough]];
-      case 5: merge_level<32>(x, tid, src, dst); [[fallthrough]];
-      case 6: merge_level<64>(x, tid, src, dst); [[fallthrough]];
-      case 7: merge_level<128>(x, tid, src, dst); [[fallthrough]];
-      case 8: merge_level<256>(x, tid, src, dst); [[fallthrough]];
-      case 9: merge_level<512>(x, tid, src, dst); [[fallthrough]];
-      default: break;
-    }
+    // the levels from runs of KP on, each unrolled for its L, until one run
+    // holds every request's keys: the pads past it are in order and below them
+    // (B = K = 4 needs 2 of its 8 levels: 4.7 us from the grid wait to the last
+    // store, 6.7 with all)
+    const int end = B * KP;
+    if (KP <= 1 && 1 < end) merge_level<1>(x, tid, src, dst);
+    if (KP <= 2 && 2 < end) merge_level<2>(x, tid, src, dst);
+    if (KP <= 4 && 4 < end) merge_level<4>(x, tid, src, dst);
+    if (KP <= 8 && 8 < end) merge_level<8>(x, tid, src, dst);
+    if (KP <= 16 && 16 < end) merge_level<16>(x, tid, src, dst);
+    if (KP <= 32 && 32 < end) merge_level<32>(x, tid, src, dst);
+    if (KP <= 64 && 64 < end) merge_level<64>(x, tid, src, dst);
+    if (KP <= 128 && 128 < end) merge_level<128>(x, tid, src, dst);
+    if (KP <= 256 && 256 < end) merge_level<256>(x, tid, src, dst);
+    if (KP <= 512 && 512 < end) merge_level<512>(x, tid, src, dst);
   } else {
     // ---- bitonic sort of the draft keys, descending ----
     x = tid < NK ? stage[(tid / RL) * RS + tid % RL] : 0ull;
