@@ -99,16 +99,24 @@ def _stream(stream):
 def _int32s(xs):
     """Host int32s for a C call: an array.array, its address in buffer_info()."""
     try:
-        return array.array("i", xs)
+        return array.array("i", iter(xs))  # iter: bytes give their values, not their storage
     except (TypeError, OverflowError):  # floats and the like: int() of each, its low 32 bits
         return array.array("i", [ctypes.c_int32(int(x)).value for x in xs])
 
 
 def _doubles(xs):
     try:
-        return array.array("d", xs)
+        return array.array("d", iter(xs))
     except TypeError:
         return array.array("d", [float(x) for x in xs])
+
+
+def _sized(a, n):
+    """a with n entries, as the C call reads: zeros follow, more are refused."""
+    if len(a) > n:
+        raise IndexError(f"{len(a)} entries for {n} candidates")
+    a.extend([0] * (n - len(a)))
+    return a
 
 
 def _check(code, where):
@@ -151,8 +159,8 @@ def spec_allocate(conf, cand_T, cand_cost, last_tokens, draft_tokens, pos_base, 
     """conf [B, K] fp32 device; cand_T / cand_cost host sequences; see spec.h."""
     B, K = conf.shape
     M = len(cand_T)
-    T = _int32s(cand_T)
-    C = _doubles(cand_cost)
+    T = _sized(_int32s(cand_T), M)
+    C = _sized(_doubles(cand_cost), M)
     code = library().spec_allocate(
         _ptr(conf), B, K, T.buffer_info()[0], C.buffer_info()[0], M, _ptr(last_tokens),
         _ptr(draft_tokens), _ptr(pos_base), _ptr(depth_out), _ptr(row_offsets_out),

@@ -251,3 +251,29 @@ def test_pointer_arguments_keep_their_checks():
     with pytest.raises(TypeError):
         spec._dtype(t.double())
     assert (spec._dtype(None), spec._dtype(t), spec._dtype(t.bfloat16())) == (spec.BF16, spec.F32, spec.BF16)
+
+
+def test_candidate_lists_of_unequal_length_are_refused():
+    """A cost list shorter than the budgets counts as zero costs, which the
+    library refuses; a longer one is refused at the binding."""
+    import pytest
+    import torch
+
+    import paper_2607_25852_gb300 as spec
+    i32, i64 = (lambda *n: torch.zeros(n, dtype=torch.int32)), (lambda *n: torch.zeros(n, dtype=torch.int64))
+
+    def call(T, C):
+        spec.spec_allocate(torch.ones(2, 3), T, C, i32(2), i32(2, 3), i64(2), i32(2), i32(3), i32(8), i64(8), i32(1),
+                           stream=_Stream0)
+
+    for C in ([], [1.0], [1.0, 2.0]):
+        with pytest.raises(spec.SpecError):
+            call([2, 4, 8], C)
+    for C in ([1.0, 2.0, 3.0, 4.0], [1.0] * 70):
+        with pytest.raises(IndexError):
+            call([2, 4, 8], C)
+    assert list(spec._int32s(b"\x04\x08")) == [4, 8] and list(spec._doubles(bytearray(8))) == [0.0] * 8
+
+
+class _Stream0:
+    cuda_stream = 0
