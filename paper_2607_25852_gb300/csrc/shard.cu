@@ -408,9 +408,8 @@ __device__ __forceinline__ void shard_level1(const ShardLaunch& p, const T* row,
       race_level1_impl<T, __nv_bfloat16, kMode, kSrcGlobalVec, kDual, true>(
           row, qrow, p.q_dtype, vend, p.v_begin, q_first, q_end, warp, kW, ra, best, best_p, p.v_begin, tail_whole);
   } else {
-    race_level1_impl<T, T, kMode, kSrcGlobalScalar, kDual, true>(row, qrow, p.q_dtype, vend, p.v_begin, q_first,
-                                                                 q_end, warp, kW, ra, best, best_p, p.v_begin,
-                                                                 tail_whole);
+    race_level1_scalar<T, kMode, kDual, true>(row, qrow, p.q_dtype, vend, p.v_begin, q_first, q_end, warp, kW, ra, best,
+                                              best_p, p.v_begin, tail_whole);
   }
 }
 

@@ -446,7 +446,7 @@ struct RaceArgs {
 };
 
 // Where level 1 reads a row from (see race_level1_impl).
-enum { kSrcGlobalVec = 0, kSrcShared = 1, kSrcGlobalScalar = 2 };
+enum { kSrcGlobalVec = 0, kSrcShared = 1 };
 
 // Raw 16-byte words of lane l's 8 entries of the four blocks of quad q
 // (entries 1024q + 256s + 8l .. +7); entries at or past V, and blocks s with
@@ -482,12 +482,11 @@ struct QuadWords {
 // Level 1 over quads [q_first, q_end) of the row, quad q to warp
 // (q - q_first) mod nwarps.  Entry indices are those of the whole vocabulary;
 // `row` (and `qrow`) address entry base_v, and entries at or past V are not
-// read.  One block is one warp step: lane l holds entries 8l..8l+7 of it
-// (kSrc 0: 16-byte loads from global memory, the whole quad's loads issued at
-// once; kSrc 1: the same from shared memory) or entries l + 32e (kSrc 2:
-// scalar loads, any layout).  The four block sums of a quad are formed
-// transposed (quad_sum): lane l races block l >> 3 of every quad, and the
-// caller takes the minimum over the lanes.
+// read.  Lane l holds entries 8l..8l+7 of each block (kSrc 0: 16-byte loads from
+// global memory, the whole quad's loads issued at once; kSrc 1: the same from
+// shared memory; race_level1_scalar takes every other layout).  The four block
+// sums of a quad are formed transposed (quad_sum): lane l races block l >> 3 of
+// every quad, and the caller takes the minimum over the lanes.
 //
 // kDual also runs the race with weights p (best_p) on the same block variates:
 // the draw a sharded caller falls back to when no shard has a positive weight.
@@ -523,47 +522,20 @@ __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype,
       raced[s] = vb < V && (!kRange || (vb >= lo && (tail_whole || vb + kRaceBlock <= V)));
     }
     float wsum[4] = {0.0f, 0.0f, 0.0f, 0.0f}, wsum_p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    uint4 r;
-    if (kSrc == kSrcGlobalScalar) {
-      r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
+    QuadWords<T, kSrc> xw;
+    QuadWords<Q, kSrc> qw;
+    xw.load(row, q, V, base_v, raced);
+    if (kMode == kWeightResidual) qw.load(qrow, q, V, base_v, raced);
+    const uint4 r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
 #pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int vb = q * kRaceQuad + s * kRaceBlock;
-        if (raced[s]) {
-          float x[8], qv[8];
+    for (int s = 0; s < 4; ++s) {
+      const int v8 = q * kRaceQuad + s * kRaceBlock + 8 * lane;
+      if (raced[s] && v8 < V) {
 #pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int v = vb + lane + 32 * e;
-            x[e] = v < V ? load_elem(static_cast<const T*>(row) + (v - base_v)) : 0.0f;
-            qv[e] = (kMode == kWeightResidual && v < V) ? load_any(qrow, q_dtype, v - base_v) : 0.0f;
-          }
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const int v = vb + lane + 32 * e;
-            if (v < V) {
-              const float ew = p_weight(x[e], a.c2, a.M2);
-              wsum[s] += weight_of<kMode>(ew, qv[e], v, a.invS, a.z_excl);
-              if (kDual) wsum_p[s] += ew;
-            }
-          }
-        }
-      }
-    } else {
-      QuadWords<T, kSrc> xw;
-      QuadWords<Q, kSrc> qw;
-      xw.load(row, q, V, base_v, raced);
-      if (kMode == kWeightResidual) qw.load(qrow, q, V, base_v, raced);
-      r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
-#pragma unroll
-      for (int s = 0; s < 4; ++s) {
-        const int v8 = q * kRaceQuad + s * kRaceBlock + 8 * lane;
-        if (raced[s] && v8 < V) {
-#pragma unroll
-          for (int e = 0; e < 8; ++e) {
-            const float ew = p_weight(xw.get(s, e), a.c2, a.M2);
-            wsum[s] += weight_of<kMode>(ew, kMode == kWeightResidual ? qw.get(s, e) : 0.0f, v8 + e, a.invS, a.z_excl);
-            if (kDual) wsum_p[s] += ew;
-          }
+        for (int e = 0; e < 8; ++e) {
+          const float ew = p_weight(xw.get(s, e), a.c2, a.M2);
+          wsum[s] += weight_of<kMode>(ew, kMode == kWeightResidual ? qw.get(s, e) : 0.0f, v8 + e, a.invS, a.z_excl);
+          if (kDual) wsum_p[s] += ew;
         }
       }
     }
@@ -580,6 +552,72 @@ __device__ __forceinline__ void race_level1(const void* row, const void* qrow, i
                                             KeyState& best) {
   race_level1_impl<T, Q, kMode, kSrc, false, false>(row, qrow, q_dtype, V, base_v, q_first, q_end, warp_id, nwarps, a,
                                                     best, best, 0, true);
+}
+
+// Level 1 of rows off the 16-byte grid, by 4-byte and 2-byte loads: a warp step
+// is one block, entries lane + 32e, so that the few blocks of a chunk spread
+// over all the CTA's warps, and a step's loads are issued before the step
+// before it is summed.  Every lane holds the same sums and the same best.  A
+// quad a warp step, its blocks' loads one after another, was bound by load
+// latency (before / now, us a call, replayed from a graph): bf16, dense q, B=2,
+// K=3, V=50001 18.8 / 10.7; B=32, K=8, V=151935 35.6 / 26.9; B=64, K=16,
+// V=100001 73.4 / 50.7; fp32, B=12, K=7, V=100003, packed 15.6 / 15.1.
+template <typename T, int kMode, bool kDual, bool kRange>
+__device__ void race_level1_scalar(const void* row, const void* qrow, int q_dtype, int V, int base_v, int q_first,
+                                   int q_end, int warp_id, int nwarps, const RaceArgs& a, KeyState& best,
+                                   KeyState& best_p, int lo, bool tail_whole) {
+  const int lane = threadIdx.x & 31;
+  float thr24 = best.key * 0x1p24f;
+  float thr24p = kDual ? best_p.key * 0x1p24f : 0.0f;
+  const int b_end = min(4 * q_end, (V + kRaceBlock - 1) / kRaceBlock);
+  float x[8], qv[8];
+  auto load = [&](int b) {
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int v = b * kRaceBlock + lane + 32 * e;
+      const bool in = v >= lo && v < V;  // a block that starts before lo is not raced
+      x[e] = in ? load_elem(static_cast<const T*>(row) + (v - base_v)) : 0.0f;
+      qv[e] = 0.0f;
+    }
+    if (kMode == kWeightResidual) {
+      auto load_q = [&](const auto* qp) {  // one branch on the type, not one a load
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          const int v = b * kRaceBlock + lane + 32 * e;
+          if (v >= lo && v < V) qv[e] = load_elem(qp + (v - base_v));
+        }
+      };
+      if (q_dtype == SPEC_F32) load_q(static_cast<const float*>(qrow));
+      else load_q(static_cast<const __nv_bfloat16*>(qrow));
+    }
+  };
+  int b = 4 * q_first + warp_id;
+  if (b < b_end) load(b);
+  for (; b < b_end; b += nwarps) {
+    const int vb = b * kRaceBlock;
+    const bool raced = !kRange || (vb >= lo && (tail_whole || vb + kRaceBlock <= V));
+    const uint4 r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)(b >> 2)), a.k0, a.k1);
+    float wsum = 0.0f, wsum_p = 0.0f;
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+      const int v = vb + lane + 32 * e;
+      if (raced && v < V) {
+        const float ew = p_weight(x[e], a.c2, a.M2);
+        wsum += weight_of<kMode>(ew, qv[e], v, a.invS, a.z_excl);
+        if (kDual) wsum_p += ew;
+      }
+    }
+    if (b + nwarps < b_end) load(b + nwarps);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+      wsum += __shfl_xor_sync(0xFFFFFFFFu, wsum, o);
+      if (kDual) wsum_p += __shfl_xor_sync(0xFFFFFFFFu, wsum_p, o);
+    }
+    const int e = b & 3;
+    const uint32_t m = race_m(e == 0 ? r.x : e == 1 ? r.y : e == 2 ? r.z : r.w);
+    race_entry(best, thr24, wsum, m, b);
+    if (kDual) race_entry(best_p, thr24p, wsum_p, m, b);
+  }
 }
 
 // Minimum key over the warp, in every lane.  Keys are positive (+inf: none, or
@@ -637,8 +675,8 @@ __device__ void race_level1_any(const VerifyLaunch& p, const void* row, const vo
       race_level1<T, __nv_bfloat16, kMode, kSrcGlobalVec>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id,
                                                           nwarps, a, best);
   } else {
-    race_level1<T, T, kMode, kSrcGlobalScalar>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id, nwarps, a,
-                                               best);
+    race_level1_scalar<T, kMode, false, false>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id, nwarps, a, best,
+                                               best, 0, true);
   }
 }
 

@@ -226,3 +226,16 @@ def test_chunked_rows(B, K, V, dtype, t):
     offs = torch.cat([torch.zeros(1, dtype=torch.int32), torch.cumsum(depth + 1, 0).to(torch.int32)])
     packed = workloads.pack_rows(wl.logits, B, K, depth)
     _check(wl, t, depth=depth, row_offsets=offs, logits=packed)
+
+
+# Rows off the 16-byte grid: one to six blocks a warp, the last block of one, of
+# 255 and of 65 entries, q of the logits' type and of the other one, q absent.
+@pytest.mark.parametrize("B,K,V,dtype", [(600, 1, 9217, "bf16"), (600, 1, 9215, "f32"), (64, 2, 40001, "bf16"),
+                                         (2, 1, 257, "f32")])
+@pytest.mark.parametrize("qmode", ["onehot", "same", "other"])
+def test_rows_off_the_grid(B, K, V, dtype, qmode):
+    wl = _random_case(V, dtype, 0.8, "onehot" if qmode == "onehot" else "dense", B=B, K=K, seed=B)
+    q = wl.q
+    if qmode == "other":
+        q = q.to(torch.float32 if dtype == "bf16" else torch.bfloat16)
+    _check(wl, 0.8, q=q)
