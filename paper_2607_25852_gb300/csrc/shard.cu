@@ -115,6 +115,7 @@ struct ShardLaunch {
   uint32_t* req_count;     // [B] arrivals per request (sample)
   int NC, chunk;           // stats: chunks per row and their length
   int NCS, quads_s, q0;    // sample: chunks, quads per chunk, first quad
+  int NCT;                 // sample: CTAs per request, NCS of them chunks
   bool vec_s;
 };
 
@@ -517,16 +518,24 @@ __device__ __forceinline__ ShardPart no_part() {
   return n;
 }
 
+// An input load issued where it stands, not sunk past the checks that follow.
+__device__ __forceinline__ uint64_t ldg_now(const uint64_t* ptr) {
+  uint64_t v;
+  asm volatile("ld.global.nc.b64 %0, [%1];" : "=l"(v) : "l"(ptr));
+  return v;
+}
+
 template <typename T>
 __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const ShardLaunch p) {
   __shared__ int sh_last, sh_b, sh_bp;
   __shared__ float sh_kb, sh_kbp;
   __shared__ KeyState sh_red[3][2 * (kSampleThreads / 32)];  // level 1, the cut blocks' parts, level 2
   __shared__ float sh_f[2 * (kSampleThreads / 32)];
-  const int i = blockIdx.x / p.NCS;
-  const int cs = blockIdx.x - i * p.NCS;
+  const int i = blockIdx.x / p.NCT;
+  const int cs = blockIdx.x - i * p.NCT;  // NCS and more: a cut block's CTA
   pdl_wait_prerequisites();
   pdl_launch_dependents();
+  const uint64_t req = ldg_now(p.request_ids + i), seed = ldg_now(p.seeds + i);  // in the record's round trip
   const ReqRec rec = p.req_rec[i];
   if (rec.flags & 1) return;  // bad input: the decision wrote the outputs
   if (rec.a < 0 || rec.a > p.K || rec.srow < 0 || rec.srow >= p.R_max || rec.z_excl < -1 || rec.z_excl >= p.V ||
@@ -540,8 +549,7 @@ __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const S
   ra.M2 = rec.M2;
   ra.invS = rec.invS;
   ra.position = rec.position;
-  ra.req = __ldg(reinterpret_cast<const unsigned long long*>(p.request_ids) + i);
-  const uint64_t seed = __ldg(reinterpret_cast<const unsigned long long*>(p.seeds) + i);
+  ra.req = req;
   ra.k0 = (uint32_t)seed;
   ra.k1 = (uint32_t)(seed >> 32);
   const int mode = (rec.flags & 4) ? kWeightResidual : (rec.flags & 2) ? kWeightExcl : kWeightP;
@@ -555,37 +563,43 @@ __global__ void __launch_bounds__(kSampleThreads, 4) shard_sample_kernel(const S
   const int q_first = p.q0 + cs * p.quads_s;
   const int q_end = min((vend + kRaceQuad - 1) / kRaceQuad, q_first + p.quads_s);
   KeyState best{INFINITY, INT_MAX}, best_p{INFINITY, INT_MAX};
-  if (mode == kWeightResidual)
-    shard_level1<T, kWeightResidual, true>(p, row, qrow, q_first, q_end, ra, best, best_p);
-  else if (mode == kWeightExcl)
-    shard_level1<T, kWeightExcl, true>(p, row, qrow, q_first, q_end, ra, best, best_p);
-  else
-    shard_level1<T, kWeightP, false>(p, row, qrow, q_first, q_end, ra, best, best_p);
-  cta_min_key2(best, best_p, sh_red[0]);
-  // ---- the cut blocks at the shard's ends: the first and the last chunk's
-  // CTA compute the shard's part of each before arriving ----
+  if (cs < p.NCS) {
+    if (mode == kWeightResidual)
+      shard_level1<T, kWeightResidual, true>(p, row, qrow, q_first, q_end, ra, best, best_p);
+    else if (mode == kWeightExcl)
+      shard_level1<T, kWeightExcl, true>(p, row, qrow, q_first, q_end, ra, best, best_p);
+    else
+      shard_level1<T, kWeightP, false>(p, row, qrow, q_first, q_end, ra, best, best_p);
+    cta_min_key2(best, best_p, sh_red[0]);
+  }
+  // ---- the cut blocks at the shard's ends: a CTA each computes the shard's
+  // part before arriving, where the grid has them, else the first and the last
+  // chunk's CTA do after their chunks (sample_ctas) ----
   const int hb = p.v_begin / kRaceBlock;   // block holding the first column
   const int tb = (vend - 1) / kRaceBlock;  // block holding the last column
   const bool head_part = p.v_begin % kRaceBlock != 0 || (vend < p.V && vend % kRaceBlock != 0 && tb == hb);
   const bool tail_part = vend < p.V && vend % kRaceBlock != 0 && tb != hb;
-  if (cs == 0 && head_part) {
+  const bool apart = p.NCT > p.NCS;
+  if (head_part && cs == (apart ? p.NCS : 0)) {
     const ShardPart pt = shard_part<T>(p, mode, row, qrow, hb, p.v_begin, tb == hb ? vend : (hb + 1) * kRaceBlock,
                                        ra, sh_red[1], sh_f);
     if (threadIdx.x == 0) p.part_ws[2 * (size_t)i] = pt;
   }
-  if (cs == p.NCS - 1 && tail_part) {
+  if (tail_part && cs == (apart ? p.NCT : p.NCS) - 1) {
     const ShardPart pt = shard_part<T>(p, mode, row, qrow, tb, tb * kRaceBlock, vend, ra, sh_red[1], sh_f);
     if (threadIdx.x == 0) p.part_ws[2 * (size_t)i + 1] = pt;
   }
   if (threadIdx.x == 0) {
-    RacePartial rp;
-    rp.key_r = best.key;
-    rp.idx_r = best.idx;
-    rp.key_p = best_p.key;
-    rp.idx_p = best_p.idx;
-    p.race_part[(size_t)i * p.NCS + cs] = rp;
+    if (cs < p.NCS) {
+      RacePartial rp;
+      rp.key_r = best.key;
+      rp.idx_r = best.idx;
+      rp.key_p = best_p.key;
+      rp.idx_p = best_p.idx;
+      p.race_part[(size_t)i * p.NCS + cs] = rp;
+    }
     __threadfence();
-    sh_last = atomicAdd(p.req_count + i, 1u) == (uint32_t)(p.NCS - 1);
+    sh_last = atomicAdd(p.req_count + i, 1u) == (uint32_t)(p.NCT - 1);
   }
   __syncthreads();
   if (!sh_last) return;
@@ -656,6 +670,20 @@ __device__ __forceinline__ uint32_t block_word(int b, const RaceArgs& a) {
   return (b & 3) == 0 ? r.x : (b & 3) == 1 ? r.y : (b & 3) == 2 ? r.z : r.w;
 }
 
+// CTAs per request for the blocks cut at the shard's ends [v_begin, v_begin + Vs)
+// of V columns: one each while the grid stays within one wave of four CTAs per
+// SM, so that a part (a row load, a race key and two CTA reductions) does not
+// follow a chunk's level 1; none past that, where CTAs of one block each would
+// only lengthen the queue.  A rank's round, replayed as a graph: B=8, K=8,
+// V=128256, rank 1 of 4 22.6 us after the chunks, 20.6 us apart; B=64, K=16,
+// V=201088, rank 3 of 8 31.6 / 31.3.
+static int sample_ctas(int B, int ncs, int v_begin, int Vs, int V) {
+  const int vend = v_begin + Vs, hb = v_begin / kRaceBlock, tb = (vend - 1) / kRaceBlock;
+  const bool tail_cut = vend < V && vend % kRaceBlock != 0;
+  const int parts = (v_begin % kRaceBlock != 0 || (tail_cut && tb == hb)) + (tail_cut && tb != hb);
+  return (long long)B * (ncs + parts) <= 152 * 4 ? parts : 0;
+}
+
 // One warp per request, a lane per shard record (more than 32 shards: in
 // turn).  A lane takes its record's whole-block keys and the cut blocks that
 // start in its shard: their parts, added in shard order, are its own part and
@@ -690,6 +718,7 @@ __global__ void __launch_bounds__(32 * kFinishWarps) shard_finish_kernel(const S
   const int i = blockIdx.x * kFinishWarps + warp;
   pdl_wait_prerequisites();
   if (i >= p.B) return;
+  const uint64_t req = ldg_now(p.request_ids + i), seed = ldg_now(p.seeds + i);  // in the record's round trip
   const ReqRec rec = p.req_rec[i];
   if (rec.flags & 1) return;  // bad input: the decision wrote the outputs
   if (rec.a < 0 || rec.a > p.K) {
@@ -698,8 +727,7 @@ __global__ void __launch_bounds__(32 * kFinishWarps) shard_finish_kernel(const S
   }
   RaceArgs a{};
   a.position = rec.position;
-  a.req = __ldg(reinterpret_cast<const unsigned long long*>(p.request_ids) + i);
-  const uint64_t seed = __ldg(reinterpret_cast<const unsigned long long*>(p.seeds) + i);
+  a.req = req;
   a.k0 = (uint32_t)seed;
   a.k1 = (uint32_t)(seed >> 32);
   FinishBest r, q;
@@ -916,7 +944,8 @@ extern "C" int spec_shard_sample(const void* logits_shard, int logits_dtype, con
   const bool q_ok = !q_shard || (spec::aligned16(q_shard) && (V_shard * qsize) % 16 == 0);
   p.vec_s = v_begin % 8 == 0 && V_shard % 8 == 0 && spec::aligned16(logits_shard) && (V_shard * esize) % 16 == 0 &&
             q_ok;
-  const unsigned grid = (unsigned)((long long)B * p.NCS);
+  p.NCT = p.NCS + spec::sample_ctas(B, p.NCS, v_begin, V_shard, V);
+  const unsigned grid = (unsigned)((long long)B * p.NCT);
   const cudaError_t err =
       logits_dtype == SPEC_F32
           ? spec::launch_after_previous(spec::shard_sample_kernel<float>, dim3(grid), dim3(spec::kSampleThreads), 0,

@@ -257,3 +257,14 @@ def test_cut_blocks(bounds, dense):
     ref = run_oracle(wl.logits, wl.drafts, wl.q, 0.9, wl.seeds, wl.request_ids, wl.pos_base)
     assert gpu["status"] == 0 and (ref["status"] == 0).all()
     compare(gpu, ref, wl.K, 0.9)
+
+
+# Cut blocks by CTAs of their own up to 608 sampling CTAs in all, by the chunks'
+# CTAs past that: one chunk and two parts a request at 202 and 203 requests (606
+# and 609), one part at the outer shards (304 and 305 requests: 608 and 610).
+@pytest.mark.parametrize("B", [202, 203, 304, 305])
+@pytest.mark.parametrize("dense", [False, True])
+def test_cut_blocks_apart_or_by_the_chunks(B, dense):
+    V = 1500
+    wl = _random_case(V, "bf16", 0.9, "dense" if dense else "onehot", B=B, K=2, seed=B)
+    _check(wl, 0.9, [0, 500, 900, V])
