@@ -48,12 +48,23 @@ static inline long long round_up(long long a, long long b) { return ceil_div(a, 
 // B=64, K=16, V=65536, t=1: 31.1 (one chunk) / 37.9; V=201088: 78.3 / 80.3;
 // B=32: 44.4 / 47.6; B=32, K=8, V=151936 with dense q: 25.2 (two chunks) /
 // 27.1; B=16, K=16, V=128256, t=0: 12.7 (two) / 13.6.
-static void stream_chunks(long long R, long long V, int& nc_out, int& chunk_out) {
+//
+// Packed rows: between B and R of them, known on the device only.  The chunks
+// then have the least sum of that cost over all rows (a light load keeps every
+// draft), half of them and a quarter, D-cut's smallest budget.  A whole step,
+// every row kept, inputs out of L2, against chunks for the quarter alone (us,
+// before / now): B=16, K=16, V=128256, t=0 31.8 / 27.7; B=32, K=8, V=151936,
+// dense q 48.1 / 42.0; V=201088, B=4 35.0 / 31.9, B=8 41.6 / 37.9, B=16 49.0 /
+// 46.3, B=32 62.8 / 64.0 (two chunks instead of four), B=64 the same; with
+// V=32768 46.2 / 43.6.  Without the half: B=32, K=8 46.1, B=16 48.4.
+static void stream_chunks(long long R, long long R_few, long long V, int& nc_out, int& chunk_out) {
   constexpr long long kRound = 16384, kSlots = 152 * 4;
   long long nc = 1, best = LLONG_MAX;
-  const long long nc_max = std::max(1LL, std::min(V / kRound, ceil_div(2 * kSlots, R)));
+  const long long nc_max = std::max(1LL, std::min(V / kRound, ceil_div(2 * kSlots, R_few)));
   for (long long n = 1; n <= nc_max; ++n) {
-    const long long cost = ceil_div(R * n, kSlots) * (ceil_div(ceil_div(V, n), kRound) + 1);
+    const long long rounds = ceil_div(ceil_div(V, n), kRound) + 1;
+    long long cost = ceil_div(R * n, kSlots) * rounds;
+    if (R_few < R) cost += (ceil_div(R_few * n, kSlots) + ceil_div(std::max(R_few, R / 2) * n, kSlots)) * rounds;
     if (cost <= best) {  // a tie takes the shorter chunks
       best = cost;
       nc = n;
@@ -70,13 +81,8 @@ static void stream_chunks(long long R, long long V, int& nc_out, int& chunk_out)
 VerifyGeometry verify_geometry(int B, int K, int V) {
   VerifyGeometry g{};
   const long long R_max = (long long)B * (K + 1);
-  stream_chunks(R_max, V, g.NC, g.chunk);
-  // Packed rows: between B and R_max of them, known on the device only.  The
-  // chunks suit a quarter of the full block, D-cut's smallest budget; for more
-  // rows they are a little short (B=64, K=16, V=201088, all rows: 1 % slower
-  // than the line above), and one chunk per row leaves a quarter of the SMs'
-  // slots empty where few are kept (272 rows of V=128256: 10 % slower).
-  stream_chunks(std::max<long long>(B, R_max / 4), V, g.NC_packed, g.chunk_packed);
+  stream_chunks(R_max, R_max, V, g.NC, g.chunk);
+  stream_chunks(R_max, std::max<long long>(B, R_max / 4), V, g.NC_packed, g.chunk_packed);
   const long long nc = std::max(g.NC, g.NC_packed);
   // Sampling pass: aim for ~560 (request, chunk) CTAs, about one resident
   // wave on 152 SMs, of >= 2048 elements each, every chunk a whole number of
