@@ -676,7 +676,8 @@ __device__ __forceinline__ uint32_t block_word(int b, const RaceArgs& a) {
 // follow a chunk's level 1; none past that, where CTAs of one block each would
 // only lengthen the queue.  A rank's round, replayed as a graph: B=8, K=8,
 // V=128256, rank 1 of 4 22.6 us after the chunks, 20.6 us apart; B=64, K=16,
-// V=201088, rank 3 of 8 31.6 / 31.3.
+// V=201088, rank 3 of 8 31.6 / 31.3.  The line at half a wave instead: rank 0
+// of those 8, one-hot q, 27.8 us against 26.8.
 static int sample_ctas(int B, int ncs, int v_begin, int Vs, int V) {
   const int vend = v_begin + Vs, hb = v_begin / kRaceBlock, tb = (vend - 1) / kRaceBlock;
   const bool tail_cut = vend < V && vend % kRaceBlock != 0;
