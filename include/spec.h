@@ -195,6 +195,9 @@ int spec_allocate(const float* conf, int B, int K, const int32_t* cand_T,
  * Arguments
  *   logits          device or host-mapped [R, V] of logits_dtype, rows of
  *                   request i at row_offsets[i] .. row_offsets[i] + n_i.
+ *                   R >= B, since every request has its row 0: with
+ *                   row_offsets, rows 0 .. B-1 may be fetched towards L2
+ *                   before the offsets are read.
  *   row_offsets     device int32 [B+1] (from spec_allocate) or NULL, meaning
  *                   row_offsets[i] = i(K+1) and R = B(K+1).
  *   depth           device int32 [B] (n_i in [0, K]) or NULL meaning n_i = K.

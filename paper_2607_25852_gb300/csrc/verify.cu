@@ -31,6 +31,7 @@
 
 #include <algorithm>
 
+#include "index_math.h"
 #include "verify_common.cuh"
 
 namespace spec {
@@ -236,30 +237,26 @@ __device__ __forceinline__ StreamItem stream_item(const VerifyLaunch& p) {
 // Before the grid-dependency wait, while the previous kernel on the stream
 // (the allocator, say: one CTA, HBM idle) drains: a line a thread of the
 // logits towards L2.  A prefetch returns no data, and L2 is where the previous
-// kernel's writes arrive, so nothing is read early.  Without row offsets it is
-// the CTA's own first load round; with them the row is not known yet, and the
-// CTAs in order take rows 0 .. B-1, which every packing holds.  Measured a call:
+// kernel's writes arrive, so nothing is read early.  stream_prefetch says which
+// entries a CTA may fetch before the depths are known.  Measured a call:
 // B=16, K=16, V=128256, t=0: 13.5 us with, 15.9 without; B=32, K=8, V=151936,
 // dense q: 27.0 / 28.4; the stress round (allocate, verify, commit): 92.2 / 93.8.
 template <typename T>
 __device__ __forceinline__ void prefetch_first_round(const VerifyLaunch& p, const StreamItem& it) {
   constexpr int kLine = 128 / (int)sizeof(T);
-  long long v, end;
-  if (p.row_offsets) {
-    v = ((long long)blockIdx.x * kStreamThreads + threadIdx.x) * kLine;
-    end = (long long)p.B * p.V;
-  } else {
-    const long long row = ((long long)it.i * (p.K + 1) + it.j) * p.V;
-    v = row + (long long)it.c * p.chunk + (long long)threadIdx.x * kLine;
-    end = row + min((long long)p.V, (long long)(it.c + 1) * p.chunk);
-  }
-  if (v < end) asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const T*>(p.logits) + v));
+  const PrefetchSpan span = stream_prefetch(p.row_offsets != nullptr, p.depth != nullptr, blockIdx.x, it.i, it.j, it.c,
+                                            p.B, p.K, p.V, p.chunk, (long long)kStreamThreads * kLine);
+  const long long v = span.first + (long long)threadIdx.x * kLine;
+  if (v < span.end) asm volatile("prefetch.global.L2 [%0];" ::"l"(static_cast<const T*>(p.logits) + v));
 }
 
 // Streaming pass with 16-byte loads from global memory (any alignment: a
-// scalar head and tail around the aligned body).
+// scalar head and tail around the aligned body).  Four CTAs of 256 threads per
+// SM, as stream_chunks counts them: left to itself the compiler may take 47
+// registers, which admits five and halves a thread's loads in flight (B=64,
+// K=16, V=201088, t=1: 82.6 us a call, 75.9 with four).
 template <typename T, bool kGreedy>
-__global__ void __launch_bounds__(kStreamThreads, kGreedy ? 4 : 0) stream_rows_kernel(const VerifyLaunch p) {
+__global__ void __launch_bounds__(kStreamThreads, 4) stream_rows_kernel(const VerifyLaunch p) {
   const StreamItem it = stream_item(p);
   prefetch_first_round<T>(p, it);
   pdl_wait_prerequisites();  // row offsets and depths come from the allocator
