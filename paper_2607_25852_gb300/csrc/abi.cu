@@ -188,8 +188,9 @@ int spec::verify_impl(const void* logits, int logits_dtype, const int32_t* row_o
   p.draft_view = reinterpret_cast<float2*>(base + g.view_off);
   p.counters = reinterpret_cast<uint32_t*>(base + g.counters_off);
   p.R_max = B * (K + 1);
-  p.NC = row_offsets ? g.NC_packed : g.NC;
-  p.chunk = row_offsets ? g.chunk_packed : g.chunk;
+  const bool fewer = row_offsets || depth;  // the call may keep fewer than B(K+1) rows
+  p.NC = fewer ? g.NC_packed : g.NC;
+  p.chunk = fewer ? g.chunk_packed : g.chunk;
   p.NCS = g.NCS;
   p.chunk_s = g.chunk_s;
   {

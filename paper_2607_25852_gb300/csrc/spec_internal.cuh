@@ -237,7 +237,7 @@ struct CommitLaunch {
 // Workspace geometry (device independent).
 struct VerifyGeometry {
   int NC, chunk;                // streaming pass, every row of the full block
-  int NC_packed, chunk_packed;  // streaming pass, packed rows (row offsets given)
+  int NC_packed, chunk_packed;  // streaming pass, as many rows as the device finds (row offsets or depths given)
   int NCS, chunk_s;
   size_t row_part_off, race_part_off, view_off, counters_off, bytes;  // [counters_off, bytes) starts at zero
 };

@@ -50,14 +50,17 @@ static inline long long round_up(long long a, long long b) { return ceil_div(a, 
 // B=32: 44.4 / 47.6; B=32, K=8, V=151936 with dense q: 25.2 (two chunks) /
 // 27.1; B=16, K=16, V=128256, t=0: 12.7 (two) / 13.6.
 //
-// Packed rows: between B and R of them, known on the device only.  The chunks
-// then have the least sum of that cost over all rows (a light load keeps every
+// Row offsets or depths: between B and R rows, known on the device only.  The
+// chunks then have the least sum of that cost over all rows (a light load keeps every
 // draft), half of them and a quarter, D-cut's smallest budget.  A whole step,
 // every row kept, inputs out of L2, against chunks for the quarter alone (us,
 // before / now): B=16, K=16, V=128256, t=0 31.8 / 27.7; B=32, K=8, V=151936,
 // dense q 48.1 / 42.0; V=201088, B=4 35.0 / 31.9, B=8 41.6 / 37.9, B=16 49.0 /
 // 46.3, B=32 62.8 / 64.0 (two chunks instead of four), B=64 the same; with
-// V=32768 46.2 / 43.6.  Without the half: B=32, K=8 46.1, B=16 48.4.
+// V=32768 46.2 / 43.6.  Without the half: B=32, K=8 46.1, B=16 48.4.  Depths in
+// the full layout, chunks for every row / so: B=64, K=16, V=201088, depths 0
+// 28.4 / 23.6, uniform 47.5 / 47.5; B=256, K=3, V=128256, depths 0 39.7 / 35.8;
+// B=16, K=16, V=128256, t=0, depths 0 5.5 / 6.0, uniform 9.5 / 8.9.
 static void stream_chunks(long long R, long long R_few, long long V, int& nc_out, int& chunk_out) {
   constexpr long long kRound = 16384, kSlots = 152 * 4;
   long long nc = 1, best = LLONG_MAX;

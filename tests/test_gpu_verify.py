@@ -239,3 +239,15 @@ def test_rows_off_the_grid(B, K, V, dtype, qmode):
     if qmode == "other":
         q = q.to(torch.float32 if dtype == "bf16" else torch.bfloat16)
     _check(wl, 0.8, q=q)
+
+
+@pytest.mark.parametrize("B,K,V", [(40, 16, 49152), (150, 3, 33000), (70, 3, 49152), (70, 3, 70000)])
+@pytest.mark.parametrize("t", [0.0, 1.0])
+def test_depths_in_the_full_layout(B, K, V, t):
+    """Rows at i(K+1) with depths from 0 to K: two to four chunks a row, where a
+    call without depths takes one or two."""
+    wl = _random_case(V, "bf16", t, "onehot", B=B, K=K, seed=B)
+    depth = torch.as_tensor(np.random.default_rng(V).integers(0, K + 1, B), dtype=torch.int32)
+    depth[:2] = torch.tensor([0, K])
+    _check(wl, t, depth=depth)
+    _check(wl, t, depth=torch.zeros_like(depth))
