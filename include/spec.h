@@ -419,9 +419,12 @@ int spec_shard_finish(const void* races, int S, const void* decisions, int B, in
  *                   logit, or a position past 2^32 - 1, sets
  *                   SPEC_ERR_BAD_INPUT; its request gets drafts -1,
  *                   confidences 0 and scores (1, 0, ..., 0).
- *   ws, ws_bytes    device workspace of at least spec_draft_workspace(B, K, V)
- *                   bytes, 256-byte aligned, zero-filled once before its first
- *                   use; left zeroed after each call.
+ *   ws, ws_bytes    device workspace of spec_draft_workspace(B, K, V) bytes,
+ *                   256-byte aligned, zero-filled once before its first use;
+ *                   each call leaves the counters in it zeroed.  The size of
+ *                   a shape serves every shape no larger in any of B, K and V;
+ *                   their counters lie elsewhere, so zero-fill it again when
+ *                   the shape changes.
  * Limits: 1 <= B, 1 <= K <= SPEC_MAX_DRAFTS, 1 <= V < SPEC_MAX_VOCAB.
  * ---------------------------------------------------------------------- */
 size_t spec_draft_workspace(int B, int K, int V);

@@ -112,6 +112,20 @@ static DraftGeometry draft_geometry(int B, int K, int V) {
   return g;
 }
 
+// Bytes that hold a call of this shape and of every smaller one.  What a shape
+// needs does not grow with each of its sizes (V = 201088, K = 1: 156,160 bytes at
+// B = 49, 103,168 at B = 64), so a workspace is asked for by a bound that does: the
+// segments of R rows are at most a wave of warps and one more a row, or as many
+// as the longest segments make of the rows, and never more than the shortest do.
+static size_t draft_workspace_bytes(int B, int K, int V) {
+  const long long R = (long long)B * K, nb = ceil_div_ll(V, 256);
+  const long long parts = std::min(R * ceil_div_ll(nb, 8),
+                                   std::max(kDraftSlots + R, R * ceil_div_ll(nb, kSegmentBlocks)));
+  const size_t bytes = ((size_t)sizeof(DraftPartial) * parts + 255) / 256 * 256 +
+                       ((size_t)sizeof(uint32_t) * (R + 2 * (size_t)B) + 255) / 256 * 256;
+  return std::max(bytes, draft_geometry(B, K, V).bytes);
+}
+
 __device__ __forceinline__ float lg2_approx(float x) {
   float y;
   asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -546,7 +560,7 @@ static cudaError_t launch_draft_typed(const DraftLaunch& p, bool vec, cudaStream
 extern "C" size_t spec_draft_workspace(int B, int K, int V) {
   if (B < 1 || K < 1 || K > SPEC_MAX_DRAFTS || V < 1 || V >= SPEC_MAX_VOCAB || (long long)B * K > (1LL << 28))
     return 0;
-  return spec::draft_geometry(B, K, V).bytes;
+  return spec::draft_workspace_bytes(B, K, V);
 }
 
 extern "C" int spec_draft(const void* logits, int logits_dtype, int B, int K, int V, float tau,

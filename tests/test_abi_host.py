@@ -277,3 +277,20 @@ def test_candidate_lists_of_unequal_length_are_refused():
 
 class _Stream0:
     cuda_stream = 0
+
+
+@pytest.mark.parametrize("entry", ["spec_draft_workspace"])
+def test_a_workspace_covers_smaller_shapes(lib, entry):
+    """An engine allocates once, for its largest batch, block and vocabulary."""
+    import paper_2607_25852_gb300 as spec
+    size = getattr(spec, entry)
+    Bs, Ks = list(range(1, 70)) + [81, 82, 100, 127, 153, 255, 256, 300, 511, 513, 700, 1117, 1300], [1, 3, 7, 8, 16, 31, 64, 255]
+    Vs = [1, 255, 1000, 4096, 8191, 8193, 16384, 25136, 32768, 50001, 65536, 128256, 151936, 201088, 1 << 20]
+    for V in Vs:
+        table = [[size(B, K, V) for K in Ks] for B in Bs]
+        for row, nxt in zip(table, table[1:]):
+            assert row == sorted(row) and all(a <= b for a, b in zip(row, nxt)), (entry, V)
+    for B in (1, 4, 16, 64, 100, 256, 600):
+        for K in Ks:
+            sizes = [size(B, K, V) for V in range(1, 260000, 1777)]
+            assert sizes == sorted(sizes), (entry, B, K)
