@@ -217,11 +217,13 @@ int spec_allocate(const float* conf, int B, int K, const int32_t* cand_T,
  *   row_stats_out   device fp32 [B(K+1), 2] or NULL: per packed row,
  *                   (max_v l/t, ln sum_v exp(l/t - max)); (max_v l, 0) at t == 0.
  *   status          device int32 [1].
- *   ws, ws_bytes    device workspace of at least spec_verify_workspace(B, K, V)
- *                   bytes, 256-byte aligned, zero-filled once before its first
- *                   use; the library leaves it zeroed again after each call.
- *                   Calls that may overlap on the device need separate
- *                   workspaces.
+ *   ws, ws_bytes    device workspace of spec_verify_workspace(B, K, V) bytes,
+ *                   256-byte aligned, zero-filled once before its first use;
+ *                   each call leaves the counters in it zeroed.  The size of
+ *                   a shape serves every shape no larger in any of B, K and V;
+ *                   their counters lie elsewhere, so zero-fill it again when
+ *                   the shape changes.  Calls that may overlap on the device
+ *                   need separate workspaces.
  * Limits: 1 <= B, 0 <= K <= SPEC_MAX_DRAFTS, 1 <= V < SPEC_MAX_VOCAB,
  * logits rows and q rows addressed with 64-bit offsets.
  * ---------------------------------------------------------------------- */
@@ -245,11 +247,10 @@ int spec_verify(const void* logits, int logits_dtype, const int32_t* row_offsets
  * Same arguments and results as spec_verify, without ws / ws_bytes: the
  * scratch is a fixed device array of SPEC_STATIC_SCRATCH_BYTES owned by the
  * library, reserved on every GPU that loads it and held until process exit.
- *   - Returns SPEC_ERR_TOO_LARGE, launching nothing, when
- *     spec_verify_workspace(B, K, V) exceeds SPEC_STATIC_SCRATCH_BYTES
- *     (4 MiB holds about 260,000 16-byte row-chunk partials; B=64, K=16,
- *     V=201088 needs spec_verify_workspace(64, 16, 201088) = 52,992
- *     bytes).
+ *   - Returns SPEC_ERR_TOO_LARGE, launching nothing, when the scratch of the
+ *     shape, at most spec_verify_workspace(B, K, V), exceeds
+ *     SPEC_STATIC_SCRATCH_BYTES (4 MiB holds about 260,000 16-byte row-chunk
+ *     partials; B=64, K=16, V=201088 needs 52,992 bytes).
  *   - The first call on a device looks up the array's device address (once
  *     per device and CUDA context, with that device current); make that
  *     first call before any stream capture.  A new context on the device

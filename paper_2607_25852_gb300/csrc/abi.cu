@@ -119,7 +119,7 @@ int spec_allocate(const float* conf, int B, int K, const int32_t* cand_T, const 
 
 size_t spec_verify_workspace(int B, int K, int V) {
   if (!verify_shape_ok(B, K, V)) return 0;
-  return spec::verify_geometry(B, K, V).bytes;
+  return spec::verify_workspace_bytes(B, K, V);
 }
 
 int spec_verify(const void* logits, int logits_dtype, const int32_t* row_offsets,

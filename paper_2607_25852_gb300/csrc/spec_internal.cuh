@@ -242,6 +242,8 @@ struct VerifyGeometry {
   size_t row_part_off, race_part_off, view_off, counters_off, bytes;  // [counters_off, bytes) starts at zero
 };
 VerifyGeometry verify_geometry(int B, int K, int V);
+size_t verify_sample_partials(int B, int V);         // a bound on B * NCS that grows with B and V
+size_t verify_workspace_bytes(int B, int K, int V);  // a bound on bytes that grows with B, K and V
 
 // Launchers (return cudaSuccess or the launch error).
 cudaError_t launch_verify(const VerifyLaunch& p, cudaStream_t stream, cudaEvent_t ev_before,

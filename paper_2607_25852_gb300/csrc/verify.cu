@@ -111,6 +111,24 @@ VerifyGeometry verify_geometry(int B, int K, int V) {
   return g;
 }
 
+// What a shape needs does not grow with each of its sizes (V = 201088, K = 16:
+// 94,976 bytes at B = 57, 52,992 at B = 64), so a workspace is asked for by a
+// bound that does: as many partials as the shortest chunks make, at most what
+// the chunks of any batch of few rows add up to, at least one a row.
+size_t verify_sample_partials(int B, int V) {  // >= B * NCS
+  return std::max<long long>(B, std::min(B * std::max(1LL, (long long)V / 2048), 559LL + 560));
+}
+size_t verify_workspace_bytes(int B, int K, int V) {
+  // R rows of NC <= 1216 / R_few + 1 chunks, and R_few >= (R - 3) / 4 rows; one
+  // chunk a row from R_few = 1216 on.  So R * NC <= 4863 * 2 below that.
+  const long long R = (long long)B * (K + 1);
+  const long long rows = std::max(R, std::min(R * std::max(1LL, (long long)V / 16384), 4863LL * 2));
+  const size_t bytes = round_up((long long)sizeof(RowPartial) * rows, 256) +
+                       round_up((long long)(sizeof(RacePartial) * verify_sample_partials(B, V)), 256) +
+                       round_up((long long)sizeof(float2) * R, 256) + round_up(sizeof(uint32_t) * (long long)B, 256);
+  return std::max(bytes, verify_geometry(B, K, V).bytes);
+}
+
 // ---------------------------------------------------------------------------
 // Decision chain (every sampling CTA at t > 0; greedy_decide_kernel at t = 0)
 // ---------------------------------------------------------------------------

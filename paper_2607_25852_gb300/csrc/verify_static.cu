@@ -97,8 +97,9 @@ extern "C" int spec_verify_static(const void* logits, int logits_dtype, const in
                                   int32_t* out_tokens, float* p_draft_out, float* row_stats_out,
                                   int32_t* status, cudaStream_t stream) {
   spec::NvtxRange range("spec_verify_static");
-  const size_t need = spec_verify_workspace(B, K, V);
-  if (need == 0) return SPEC_ERR_INVALID_ARG;
+  if (spec_verify_workspace(B, K, V) == 0) return SPEC_ERR_INVALID_ARG;
+  const spec::VerifyGeometry g = spec::verify_geometry(B, K, V);
+  const size_t need = g.bytes;  // this shape's own layout, no more
   if (need > (size_t)SPEC_STATIC_SCRATCH_BYTES) return SPEC_ERR_TOO_LARGE;
   void* scratch = nullptr;
   const int rc = scratch_address(&scratch);
@@ -107,7 +108,6 @@ extern "C" int spec_verify_static(const void* logits, int logits_dtype, const in
   // than rely on what the previous call left behind.  The clear is queued
   // only after spec_verify's argument checks, so a rejected call leaves the
   // stream and the scratch untouched.
-  const spec::VerifyGeometry g = spec::verify_geometry(B, K, V);
   ClearRange clear{static_cast<char*>(scratch) + g.counters_off, need - g.counters_off};
   return spec::verify_impl(logits, logits_dtype, row_offsets, depth, draft_tokens, q, q_dtype, B, K, V,
                            temperature, seeds, request_ids, pos_base, accepted_len_out, out_tokens, p_draft_out,
