@@ -326,9 +326,11 @@ int spec_commit(const int32_t* accepted_len, const int32_t* out_tokens,
 #define SPEC_SHARD_RACE_BYTES 96     /* per (shard, request) */
 
 /* Workspace of spec_shard_stats and spec_shard_sample on one rank: 256-byte
- * aligned, zero-filled once before its first use, left zeroed by every call;
- * calls that may overlap on the device need separate workspaces.  0 for an
- * invalid shape. */
+ * aligned, zero-filled once before its first use; every call leaves the counters
+ * in it zeroed.  The size of a shape serves every shape no larger in any of B, K
+ * and V_shard; their counters lie elsewhere, so zero-fill it again when the shape
+ * changes.  Calls that may overlap on the device need separate workspaces.  0 for
+ * an invalid shape. */
 size_t spec_shard_workspace(int B, int K, int V_shard);
 
 /* spec_shard_stats -- per packed row, over the shard's columns: (max, sum of

@@ -155,6 +155,21 @@ static ShardGeometry shard_geometry(int B, int K, int Vs) {
   return s;
 }
 
+// As verify_workspace_bytes: a bound that grows with B, K and Vs (what a shape
+// needs does not: K = 64, Vs = 65536 92,928 bytes at B = 20, 92,416 at B = 36).
+// R rows of at most 4095 / R + 1 chunks, one a row from R = 4096 on; a shard's
+// sampling chunks are at most one more a request than a vocabulary's, and hold
+// at least eight quads.
+static size_t shard_workspace_bytes(int B, int K, int Vs) {
+  const long long R = (long long)B * (K + 1);
+  const long long rows = std::max(R, std::min(R * std::max(1LL, (long long)Vs / 16384), 4095LL * 2));
+  const long long nq_max = (Vs + kRaceQuad - 1) / kRaceQuad + 1;
+  const long long races = std::min(B * ((nq_max + 7) / 8), (long long)verify_sample_partials(B, Vs) + B);
+  const size_t bytes = round256(sizeof(RowPartial) * rows) + round256(sizeof(RacePartial) * races) +
+                       round256(sizeof(ShardPart) * 2 * (size_t)B) + round256(sizeof(uint32_t) * (size_t)(R + B));
+  return std::max(bytes, shard_geometry(B, K, Vs).bytes);
+}
+
 // ---------------------------------------------------------------------------
 // spec_shard_stats: one CTA per (request, row, chunk of the shard); the last
 // CTA of a row to finish merges the row's chunk partials into its record.
@@ -805,7 +820,7 @@ extern "C" size_t spec_shard_workspace(int B, int K, int V_shard) {
   if (B < 1 || K < 0 || K > SPEC_MAX_DRAFTS || V_shard < 1 || V_shard >= SPEC_MAX_VOCAB ||
       (long long)B * (K + 1) > (1LL << 28))
     return 0;
-  return spec::shard_geometry(B, K, V_shard).bytes;
+  return spec::shard_workspace_bytes(B, K, V_shard);
 }
 
 extern "C" int spec_shard_stats(const void* logits_shard, int logits_dtype, const int32_t* row_offsets,

@@ -279,7 +279,7 @@ class _Stream0:
     cuda_stream = 0
 
 
-@pytest.mark.parametrize("entry", ["spec_draft_workspace", "spec_verify_workspace"])
+@pytest.mark.parametrize("entry", ["spec_draft_workspace", "spec_verify_workspace", "spec_shard_workspace"])
 def test_a_workspace_covers_smaller_shapes(lib, entry):
     """An engine allocates once, for its largest batch, block and vocabulary."""
     import paper_2607_25852_gb300 as spec
