@@ -43,4 +43,28 @@ SPEC_HD PrefetchSpan stream_prefetch(bool packed, bool has_depth, int block, int
   return PrefetchSpan{row + c * chunk, row + (last < V ? last : V)};
 }
 
+// The units of U that the Markov head's U producer loads, in its order of issue
+// u = 0, 1, ..: a tile's 64 rows x 128 columns when the operand's rows are
+// repeated (dup), else one 64-column half of a tile, the halves in turn.  Tile t
+// belongs to epilogue group t % halves; unit m of a group uses one of the group's
+// `depth` stages in turn, so that a stage's phases are seen one after another.
+struct UnitsOfU {
+  bool dup;
+  int halves, depth;
+  SPEC_HD int per_tile() const { return dup ? 1 : 2; }
+  SPEC_HD int tile(int u) const { return dup ? u : u >> 1; }
+  SPEC_HD int m(int u) const { return tile(u) / halves * per_tile() + (dup ? 0 : (u & 1)); }
+  SPEC_HD int stage(int u) const { return tile(u) % halves + halves * (m(u) % depth); }
+  SPEC_HD unsigned parity(int u) const { return (unsigned)(m(u) / depth) & 1u; }
+  // The unit that takes u's stage after it.
+  SPEC_HD int next(int u) const {
+    const int later = m(u) + depth, t = tile(u) % halves + halves * (later / per_tile());
+    return per_tile() * t + (dup ? 0 : (later & 1));
+  }
+  // Giving up after `issued` units: does the producer wait for unit u to land?
+  // Only for the last one of its stage, whose parity the barrier still shows; a
+  // wait for an earlier one would run to its limit.
+  SPEC_HD bool drains(int u, int issued) const { return u < issued && next(u) >= issued; }
+};
+
 }  // namespace spec

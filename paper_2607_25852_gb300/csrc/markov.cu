@@ -63,6 +63,7 @@
 
 #include <algorithm>
 
+#include "index_math.h"
 #include "verify_common.cuh"
 
 namespace spec {
@@ -431,13 +432,13 @@ __global__ void __launch_bounds__(kMkThreads, 1)
     if (lane == 0) {
       asm volatile("prefetch.tensormap [%0];" ::"l"(reinterpret_cast<uint64_t>(&tmU)) : "memory");
       const uint64_t once = evict_first_policy();
-      const int per = dup ? 1 : 2;  // units per tile
-      auto unit_m = [&](int u) { return ((dup ? u : u >> 1) / kMkHalves) * per + (dup ? 0 : (u & 1)); };
-      auto unit_stage = [&](int u) { return (dup ? u : u >> 1) % kMkHalves + kMkHalves * (unit_m(u) % p.u_depth); };
+      const UnitsOfU units{dup, kMkHalves, p.u_depth};
+      const int n = T * units.per_tile();
       int u = 0;
-      for (; u < T * per; ++u) {
-        const int t = dup ? u : u >> 1, m = unit_m(u), st = unit_stage(u);
-        if (m >= p.u_depth && !mbar_wait(&bar_ufree[st], (uint32_t)((m / p.u_depth - 1) & 1), p.status)) abort_sh = 1;
+      for (; u < n; ++u) {
+        const int t = units.tile(u), m = units.m(u), st = units.stage(u);
+        // the stage's previous unit has been read: its phase is the one before
+        if (m >= p.u_depth && !mbar_wait(&bar_ufree[st], units.parity(u) ^ 1u, p.status)) abort_sh = 1;
         if (abort_sh) break;
         const int v0 = ((int)blockIdx.x + t * p.G) * kMkTile;
         uint8_t* dst = sU + st * kMkUBytes;
@@ -451,9 +452,9 @@ __global__ void __launch_bounds__(kMkThreads, 1)
         }
       }
       // given up: what is still in flight lands before the CTA leaves
-      if (u < T * per)
-        for (int x = max(0, u - 2 * kMkHalves * p.u_depth); x < u; ++x)
-          mbar_wait(&bar_ufull[unit_stage(x)], (uint32_t)((unit_m(x) / p.u_depth) & 1), p.status);
+      if (u < n)
+        for (int x = 0; x < u; ++x)
+          if (units.drains(x, u)) mbar_wait(&bar_ufull[units.stage(x)], units.parity(x), p.status);
     }
     __syncwarp();
   } else if (epi_active) {

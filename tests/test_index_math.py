@@ -18,6 +18,16 @@ void stream_prefetch(int packed, int has_depth, int block, int i, int j, int c, 
   out[0] = s.first;
   out[1] = s.end;
 }
+void unit_of_u(int dup, int halves, int depth, int u, int* out) {
+  const spec::UnitsOfU x{dup != 0, halves, depth};
+  out[0] = x.tile(u);
+  out[1] = x.m(u);
+  out[2] = x.stage(u);
+  out[3] = (int)x.parity(u);
+}
+int unit_drains(int dup, int halves, int depth, int u, int issued) {
+  return spec::UnitsOfU{dup != 0, halves, depth}.drains(u, issued);
+}
 }
 """
 
@@ -56,3 +66,27 @@ def test_prefetched_entries_are_kept_rows(lib, B, K, V, chunk, packed, has_depth
         else:
             row = (i * (K + 1) + j) * V
             assert first == row + c * chunk and end == min(row + V, row + (c + 1) * chunk, first + per)
+
+
+@pytest.mark.parametrize("dup", [True, False])
+@pytest.mark.parametrize("depth", [1, 2, 3])
+def test_units_of_u_wait_on_the_last_phase_of_a_stage(lib, dup, depth):
+    """A stage's barrier completes one phase a unit, and a parity wait sees only
+    the last one: the producer's waits must each be for a stage's last unit
+    (an earlier one would never be seen), and all of them for every stage in
+    use.  Units before the ring wraps have parity 0, and tiles go to the two
+    epilogue groups in turn."""
+    halves = 2
+    unit = (ctypes.c_int * 4)()
+    for issued in range(0, 12 * halves * depth + 3):
+        phases, waits = {}, []
+        for u in range(issued):
+            lib.unit_of_u(int(dup), halves, depth, u, unit)
+            tile, m, stage, parity = unit
+            assert tile == (u if dup else u // 2) and stage % halves == tile % halves
+            assert parity == phases.get(stage, 0) % 2 and 0 <= stage < halves * depth
+            phases[stage] = phases.get(stage, 0) + 1
+            if lib.unit_drains(int(dup), halves, depth, u, issued):
+                waits.append((stage, parity))
+        assert sorted(s for s, _ in waits) == sorted(phases)
+        assert all(parity == (phases[stage] - 1) % 2 for stage, parity in waits)
