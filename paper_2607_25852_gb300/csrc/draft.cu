@@ -18,7 +18,7 @@
 // 2^(l*c2 - fl(M_r*c2)) needs three shuffles inside its lane group; the
 // round's max M_r comes from one redux over order-preserving integer keys.
 // Level 1 of the race compares blocks in the log2 domain,
-//   log2 key_b = log2 E_b - log2 sum_b - M_r*c2   (see BlockKey),
+//   log2 key_b = log2 E_b - log2 sum_b - fl(M_r*c2)   (see BlockKey),
 // so no pass over the row is needed before the draw.  Each lane keeps the sum
 // of one block of every 32, forms that block's key once, and holds its own
 // best block and its own part of the softmax sum until the segment ends: no
@@ -42,18 +42,19 @@ constexpr int kDraftSlots = 152 * kDraftCtas * kDraftThreads / 32;  // warps in 
 constexpr int kSegmentBlocks = 64;  // race blocks per warp unit, at most
 constexpr int kGroup = 32;          // race blocks whose level-1 words one warp-wide Philox call gives
 
-// A level-1 candidate: block idx with L = log2 E_b - log2 sum_b and block
-// max M, i.e. log2 key = L - M*c2.  Two candidates compare by
-// L_a - L_b < c2 * (M_a - M_b): the rounding then scales with the gap between
-// the two maxima, not with |M*c2| (which reaches hundreds at small tau).
+// A level-1 candidate: block idx with L = log2 E_b - log2 sum_b and P =
+// fl(M_r*c2), to which sum_b is relative: log2 key = L - P.  Two candidates
+// compare by L_a - L_b < P_a - P_b: the rounding of |M*c2|, which reaches
+// thousands at small tau, is in the sum and in P alike and cancels, and the
+// difference of two P rounds with the gap between them.
 struct BlockKey {
-  float L, M;
+  float L, P;
   int32_t idx;  // INT_MAX: none
 };
-__device__ __forceinline__ bool block_key_better(const BlockKey& a, const BlockKey& b, float c2) {
+__device__ __forceinline__ bool block_key_better(const BlockKey& a, const BlockKey& b) {
   if (a.idx == INT_MAX) return false;
   if (b.idx == INT_MAX) return true;
-  const float lhs = a.L - b.L, rhs = c2 * (a.M - b.M);
+  const float lhs = a.L - b.L, rhs = a.P - b.P;
   return lhs < rhs || (lhs == rhs && a.idx < b.idx);
 }
 
@@ -63,7 +64,7 @@ struct alignas(16) DraftPartial {
   float key;      // tau > 0: L of the best block; tau = 0: the max (= m)
   int32_t idx;    // tau > 0: the best block; tau = 0: first block of the first round that holds the max (INT_MAX: none)
   int32_t flags;  // bit0: NaN or +inf seen
-  float keyM;     // tau > 0: M of the best block
+  float keyP;     // tau > 0: P of the best block
   int32_t pad[2];
 };
 
@@ -244,7 +245,7 @@ struct WarpDraftState {
   float m = -INFINITY, s = 0.0f;           // max, and the lane's sum of 2^(l*c2 - fl(m*c2)); NaN once a NaN or +inf was read
   BlockKey best{INFINITY, 0.0f, INT_MAX};  // tau > 0: the best of the lane's blocks
   int32_t first = INT_MAX;                 // tau = 0: first block of the first round that reaches m
-  float keep_s = 0.0f, keep_m = 0.0f;      // tau > 0: the lane's block of the current 32: its sum, relative to keep_m
+  float keep_s = 0.0f, keep_p = 0.0f;      // tau > 0: the lane's block of the current 32: its sum, and P
 };
 
 // The lane's block among each 32 (level 1 of the race): the round whose index
@@ -322,18 +323,19 @@ __device__ __forceinline__ void draft_round(WarpDraftState& ws, const uint4 (&w)
   const float sb = block_sum(acc, lane);
   if (((b0 & (kGroup - 1)) / R::kBlocks) == owned_round<T>(lane)) {
     ws.keep_s = sb;
-    ws.keep_m = Mr;
+    ws.keep_p = M2;
   }
 }
 
 // Level-1 key of the lane's block `b` once its round is in (b < b_hi).
-__device__ __forceinline__ void draft_candidate(WarpDraftState& ws, int b, uint32_t word, float c2) {
-  // E near 0 needs log1pf; log2 of E and of the sum go to lg2.approx, whose
-  // absolute error (~1e-7) is what a log-domain key can afford
+__device__ __forceinline__ void draft_candidate(WarpDraftState& ws, int b, uint32_t word) {
+  // E near 0 needs log1pf; log2 of E and of the sum go to lg2.approx: its error,
+  // 2^-22 of the result (absolute next to 1), is at most 6e-6 at E = 2^-24, the
+  // least there is, and 2e-6 at the E of a typical winner
   if (!(ws.keep_s > 0.0f)) return;
   const float E = -log1pf(-((float)race_m(word) * 0x1p-24f));
-  const BlockKey k{lg2_approx(E) - lg2_approx(ws.keep_s), ws.keep_m, b};
-  if (block_key_better(k, ws.best, c2)) ws.best = k;
+  const BlockKey k{lg2_approx(E) - lg2_approx(ws.keep_s), ws.keep_p, b};
+  if (block_key_better(k, ws.best)) ws.best = k;
 }
 
 // One warp per (row, segment of blocks); the warps of a CTA are independent
@@ -385,7 +387,7 @@ __global__ void __launch_bounds__(kDraftThreads, kDraftCtas) draft_rows_kernel(c
     draft_round<T, kGreedy>(ws, w, b0, lane, p.c2);
     const int bn = b0 + R::kBlocks;
     if (!kGreedy && (bn >= b_hi || (bn & (kGroup - 1)) == 0))
-      draft_candidate(ws, (b0 & ~(kGroup - 1)) + owned_block<T>(lane), word, p.c2);
+      draft_candidate(ws, (b0 & ~(kGroup - 1)) + owned_block<T>(lane), word);
   }
 
   // ---- the segment's partial over the lanes; the last warp of the row goes on ----
@@ -393,9 +395,9 @@ __global__ void __launch_bounds__(kDraftThreads, kDraftCtas) draft_rows_kernel(c
   for (int o = 16; o > 0; o >>= 1) {
     ws.s += __shfl_xor_sync(0xFFFFFFFFu, ws.s, o);
     if (!kGreedy) {
-      const BlockKey ob{__shfl_xor_sync(0xFFFFFFFFu, ws.best.L, o), __shfl_xor_sync(0xFFFFFFFFu, ws.best.M, o),
+      const BlockKey ob{__shfl_xor_sync(0xFFFFFFFFu, ws.best.L, o), __shfl_xor_sync(0xFFFFFFFFu, ws.best.P, o),
                         __shfl_xor_sync(0xFFFFFFFFu, ws.best.idx, o)};
-      if (block_key_better(ob, ws.best, p.c2)) ws.best = ob;
+      if (block_key_better(ob, ws.best)) ws.best = ob;
     }
   }
   int last = 0;
@@ -404,7 +406,7 @@ __global__ void __launch_bounds__(kDraftThreads, kDraftCtas) draft_rows_kernel(c
     d.m = ws.m;
     d.s = ws.s;
     d.key = kGreedy ? ws.m : ws.best.L;
-    d.keyM = kGreedy ? 0.0f : ws.best.M;
+    d.keyP = kGreedy ? 0.0f : ws.best.P;
     d.idx = kGreedy ? ws.first : ws.best.idx;
     d.flags = ws.s != ws.s;
     p.part[(size_t)r * p.NC + c] = d;
@@ -429,7 +431,7 @@ __global__ void __launch_bounds__(kDraftThreads, kDraftCtas) draft_rows_kernel(c
       if (arg_better(o, g)) g = o;
     } else {
       const BlockKey o{__uint_as_float(a.z), __uint_as_float(b2.y), (int32_t)a.w};
-      if (block_key_better(o, best, p.c2)) best = o;
+      if (block_key_better(o, best)) best = o;
     }
     f |= (int32_t)b2.x;
   }
@@ -437,9 +439,9 @@ __global__ void __launch_bounds__(kDraftThreads, kDraftCtas) draft_rows_kernel(c
   for (int o = 16; o > 0; o >>= 1) {
     st = soft_merge(st, SoftState{__shfl_xor_sync(0xFFFFFFFFu, st.m, o), __shfl_xor_sync(0xFFFFFFFFu, st.s, o)},
                     p.c2);
-    const BlockKey ob{__shfl_xor_sync(0xFFFFFFFFu, best.L, o), __shfl_xor_sync(0xFFFFFFFFu, best.M, o),
+    const BlockKey ob{__shfl_xor_sync(0xFFFFFFFFu, best.L, o), __shfl_xor_sync(0xFFFFFFFFu, best.P, o),
                       __shfl_xor_sync(0xFFFFFFFFu, best.idx, o)};
-    if (block_key_better(ob, best, p.c2)) best = ob;
+    if (block_key_better(ob, best)) best = ob;
     const ArgState og{__shfl_xor_sync(0xFFFFFFFFu, g.v, o), __shfl_xor_sync(0xFFFFFFFFu, g.idx, o)};
     if (arg_better(og, g)) g = og;
   }
