@@ -708,7 +708,7 @@ __global__ void __launch_bounds__(kPickThreads, 1) markov_pick_kernel(const Mark
   const float M2 = __fmul_rn(M, p.c2);
 
   // ---- the row's sum; level 1 (tau > 0): log2 key of every 256-entry block,
-  // log2 E_b - log2 sum_b + c2 (M - m_b), one block a thread; at tau = 0 the
+  // log2 E_b - log2 sum_b + fl(M c2) - fl(m_b c2), one block a thread; at tau = 0 the
   // lowest index that attains the max ----
   {
     float s = st.m > -INFINITY ? st.s * exp2f(__fmul_rn(st.m, p.c2) - M2) : st.s;
@@ -734,7 +734,7 @@ __global__ void __launch_bounds__(kPickThreads, 1) markov_pick_kernel(const Mark
           if (left > 1) bs += sq0.w * ex2_approx(__fmul_rn(m1, p.c2) - b2);
           if (left > 2) bs += sq1.y * ex2_approx(__fmul_rn(m2, p.c2) - b2);
           if (left > 3) bs += sq1.w * ex2_approx(__fmul_rn(m3, p.c2) - b2);
-          const float k = lgE - mk_lg2(bs) + p.c2 * (M - bm);
+          const float k = lgE - mk_lg2(bs) + (M2 - b2);  // the products that the sums are relative to
           if (bs > 0.0f && k < key) {  // b increases: a tie keeps the lower block
             key = k;
             idx = b;

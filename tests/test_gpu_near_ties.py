@@ -7,6 +7,7 @@ import torch
 
 import near_ties
 from test_gpu_draft import run_draft, run_oracle_draft
+from test_gpu_markov import run_markov
 
 pytestmark = pytest.mark.gpu
 
@@ -27,5 +28,16 @@ def test_draft(dtype, V, a, b):
     want = run_oracle_draft(logits, float(near_ties.TAU), *requests)["z"][:, 0]
     assert (want // 256).tolist() == winner.tolist()
     got = run_draft(logits.to(dtype), float(near_ties.TAU), *requests)
+    assert got["status"] == 0
+    assert (got["z"][:, 0] // 256).tolist() == winner.tolist()
+
+
+@pytest.mark.parametrize("V,a,b", [(1024, 0, 2), (4096, 14, 3), (5000, 18, 2)])
+def test_markov(V, a, b):
+    """W1 = 0, so that the logits are U exactly."""
+    logits, requests, winner = _case(V, a, b, limit=128)
+    B = len(winner)
+    zero = torch.zeros((V, 64), dtype=torch.bfloat16)
+    got = run_markov(logits, zero, zero.t(), torch.zeros(B, dtype=torch.int32), float(near_ties.TAU), *requests)
     assert got["status"] == 0
     assert (got["z"][:, 0] // 256).tolist() == winner.tolist()
