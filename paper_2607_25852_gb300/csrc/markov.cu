@@ -687,15 +687,17 @@ __global__ void __launch_bounds__(kPickThreads, 1) markov_pick_kernel(const Mark
   ArgState g{-INFINITY, INT_MAX};
   const int n = kMkParts * p.G;
   const uint4* src = reinterpret_cast<const uint4*>(p.part + (size_t)i * n);
+  uint32_t flagged = 0;
   for (int c = threadIdx.x; c < n; c += kPickThreads) {
     const uint4 lo = __ldcg(src + 2 * c), hi = __ldcg(src + 2 * c + 1);
     st = soft_merge(st, SoftState{__uint_as_float(lo.x), __uint_as_float(lo.y)}, p.c2);
-    if (hi.y) st.s = NAN;  // a NaN or +inf entry: the sum marks the row
+    flagged |= hi.y;
     if (kGreedy) {
       const ArgState a{__uint_as_float(lo.z), (int)lo.w};
       if (arg_better(a, g)) g = a;
     }
   }
+  if (flagged) st.s = NAN;  // a NaN or +inf entry: the sum marks the row, once no other state is merged into it
 
   // ---- the row's max ----
   {
