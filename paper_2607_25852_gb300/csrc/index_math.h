@@ -36,11 +36,17 @@ struct PrefetchSpan {
 //   V=128256, every row kept, 64.8 us a call with every CTA fetching, 63.2 so.
 SPEC_HD PrefetchSpan stream_prefetch(bool packed, bool has_depth, int block, int i, int j, int c, int B, int K,
                                      long long V, long long chunk, long long per_cta) {
-  if (packed) return PrefetchSpan{block * per_cta, block < kStreamWave ? B * V : 0};
-  if (has_depth && j > 0) return PrefetchSpan{0, 0};
-  const long long row = ((long long)i * (K + 1) + j) * V;
-  const long long last = (c + 1) * chunk;
-  return PrefetchSpan{row + c * chunk, row + (last < V ? last : V)};
+  PrefetchSpan s;
+  if (packed) {
+    const long long wave = kStreamWave * per_cta;
+    s.first = block * per_cta;
+    s.end = B * V < wave ? B * V : wave;
+  } else {
+    const long long row = ((long long)i * (K + 1) + j) * V, last = (c + 1) * chunk;
+    s.first = row + c * chunk;
+    s.end = has_depth && j > 0 ? 0 : row + (V < last ? V : last);
+  }
+  return s;
 }
 
 // The units of U that the Markov head's U producer loads, in its order of issue
