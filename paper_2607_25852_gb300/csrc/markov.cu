@@ -169,6 +169,14 @@ __device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, int32_
   return mbar_try_wait(bar, parity) || mbar_wait_slow(bar, parity, status);
 }
 
+__device__ __forceinline__ uint4 lds16(const void* ptr) {
+  uint4 v;
+  asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
+               : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
+               : "r"(smem_u32(ptr)));
+  return v;
+}
+
 __device__ __forceinline__ void tma_load_2d(void* dst, const CUtensorMap* map, int x, int y, uint64_t* bar) {
   asm volatile(
       "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];" ::
@@ -484,7 +492,7 @@ __global__ void __launch_bounds__(kMkThreads, 1)
       if (!__all_sync(0xFFFFFFFFu, mbar_wait(&bar_ufull[st], (uint32_t)((s / p.u_depth) & 1), p.status))) return false;
       const uint8_t* src = sU + st * kMkUBytes + (dup ? col_half * (kMkUBytes / 2) : 0) + row * 128;
 #pragma unroll
-      for (int j = 0; j < 8; ++j) uw[j] = load16<true>(src + ((j ^ (row & 7)) << 4));
+      for (int j = 0; j < 8; ++j) uw[j] = lds16(src + ((j ^ (row & 7)) << 4));
       __syncwarp();
       if (lane == 0) mbar_arrive(&bar_ufree[st]);
       // columns past V read 0 through the tensor map: -inf instead (V % 8 == 0)

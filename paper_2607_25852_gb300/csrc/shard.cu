@@ -417,11 +417,11 @@ __device__ __forceinline__ void shard_level1(const ShardLaunch& p, const T* row,
   constexpr int kW = kSampleThreads / 32;
   if (p.vec_s) {
     if (kMode == kWeightResidual && p.q_dtype == SPEC_F32)
-      race_level1_impl<T, float, kMode, kSrcGlobalVec, kDual, true>(row, qrow, p.q_dtype, vend, p.v_begin, q_first,
+      race_level1_impl<T, float, kMode, kDual, true>(row, qrow, p.q_dtype, vend, p.v_begin, q_first,
                                                                     q_end, warp, kW, ra, best, best_p, p.v_begin,
                                                                     tail_whole);
     else
-      race_level1_impl<T, __nv_bfloat16, kMode, kSrcGlobalVec, kDual, true>(
+      race_level1_impl<T, __nv_bfloat16, kMode, kDual, true>(
           row, qrow, p.q_dtype, vend, p.v_begin, q_first, q_end, warp, kW, ra, best, best_p, p.v_begin, tail_whole);
   } else {
     race_level1_scalar<T, kMode, kDual, true>(row, qrow, p.q_dtype, vend, p.v_begin, q_first, q_end, warp, kW, ra, best,

@@ -336,54 +336,6 @@ __device__ __forceinline__ RowPartial cta_reduce_partial(RowAcc<T, kGreedy>& acc
 // ---------------------------------------------------------------------------
 // Sampling pass (t > 0)
 // ---------------------------------------------------------------------------
-// Eight consecutive entries of a row as floats, from 16-byte loads: from
-// global memory (streaming) or from a chunk staged in shared memory.
-template <bool kShared>
-__device__ __forceinline__ uint4 load16(const void* ptr) {
-  if (kShared) {
-    uint4 v;
-    asm volatile("ld.shared.v4.u32 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(v.x), "=r"(v.y), "=r"(v.z), "=r"(v.w)
-                 : "r"((uint32_t)__cvta_generic_to_shared(ptr)));
-    return v;
-  }
-  return ldg_stream(ptr);
-}
-
-template <typename T>
-struct Row8;
-template <>
-struct Row8<__nv_bfloat16> {
-  template <bool kShared>
-  __device__ static void load(const void* row, int g8, float x[8]) {
-    const uint4 w = load16<kShared>(static_cast<const uint4*>(row) + g8);
-    x[0] = bf16_lo(w.x);
-    x[1] = bf16_hi(w.x);
-    x[2] = bf16_lo(w.y);
-    x[3] = bf16_hi(w.y);
-    x[4] = bf16_lo(w.z);
-    x[5] = bf16_hi(w.z);
-    x[6] = bf16_lo(w.w);
-    x[7] = bf16_hi(w.w);
-  }
-};
-template <>
-struct Row8<float> {
-  template <bool kShared>
-  __device__ static void load(const void* row, int g8, float x[8]) {
-    const uint4 a = load16<kShared>(static_cast<const uint4*>(row) + 2 * g8);
-    const uint4 b = load16<kShared>(static_cast<const uint4*>(row) + 2 * g8 + 1);
-    x[0] = __uint_as_float(a.x);
-    x[1] = __uint_as_float(a.y);
-    x[2] = __uint_as_float(a.z);
-    x[3] = __uint_as_float(a.w);
-    x[4] = __uint_as_float(b.x);
-    x[5] = __uint_as_float(b.y);
-    x[6] = __uint_as_float(b.z);
-    x[7] = __uint_as_float(b.w);
-  }
-};
-
 // ---------------------------------------------------------------------------
 // Two-level exponential race
 // ---------------------------------------------------------------------------
@@ -445,13 +397,10 @@ struct RaceArgs {
   uint32_t k0, k1;
 };
 
-// Where level 1 reads a row from (see race_level1_impl).
-enum { kSrcGlobalVec = 0, kSrcShared = 1 };
-
 // Raw 16-byte words of lane l's 8 entries of the four blocks of quad q
 // (entries 1024q + 256s + 8l .. +7); entries at or past V, and blocks s with
 // raced[s] false, are not read.
-template <typename E, int kSrc>
+template <typename E>
 struct QuadWords {
   static constexpr int kWords = sizeof(E) == 4 ? 2 : 1;  // 16-byte words per 8 entries
   uint4 w[4][kWords];
@@ -463,7 +412,7 @@ struct QuadWords {
 #pragma unroll
       for (int h = 0; h < kWords; ++h)
         w[s][h] = raced[s] && v8 < V
-                      ? load16<kSrc == kSrcShared>(static_cast<const uint4*>(base) + (((v8 - base_v) >> 3) * kWords + h))
+                      ? ldg_stream(static_cast<const uint4*>(base) + (((v8 - base_v) >> 3) * kWords + h))
                       : make_uint4(0u, 0u, 0u, 0u);
     }
   }
@@ -482,9 +431,8 @@ struct QuadWords {
 // Level 1 over quads [q_first, q_end) of the row, quad q to warp
 // (q - q_first) mod nwarps.  Entry indices are those of the whole vocabulary;
 // `row` (and `qrow`) address entry base_v, and entries at or past V are not
-// read.  Lane l holds entries 8l..8l+7 of each block (kSrc 0: 16-byte loads from
-// global memory, the whole quad's loads issued at once; kSrc 1: the same from
-// shared memory; race_level1_scalar takes every other layout).  The four block
+// read.  Lane l holds entries 8l..8l+7 of each block, by 16-byte loads, the whole
+// quad's issued at once (race_level1_scalar takes rows off that grid).  The four block
 // sums of a quad are formed transposed (quad_sum): lane l races block l >> 3 of
 // every quad, and the caller takes the minimum over the lanes.
 //
@@ -507,7 +455,7 @@ __device__ __forceinline__ float quad_sum(const float (&w)[4], int lane) {
   return v;
 }
 
-template <typename T, typename Q, int kMode, int kSrc, bool kDual, bool kRange>
+template <typename T, typename Q, int kMode, bool kDual, bool kRange>
 __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype, int V, int base_v, int q_first,
                                  int q_end, int warp_id, int nwarps, const RaceArgs& a, KeyState& best,
                                  KeyState& best_p, int lo, bool tail_whole) {
@@ -522,8 +470,8 @@ __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype,
       raced[s] = vb < V && (!kRange || (vb >= lo && (tail_whole || vb + kRaceBlock <= V)));
     }
     float wsum[4] = {0.0f, 0.0f, 0.0f, 0.0f}, wsum_p[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-    QuadWords<T, kSrc> xw;
-    QuadWords<Q, kSrc> qw;
+    QuadWords<T> xw;
+    QuadWords<Q> qw;
     xw.load(row, q, V, base_v, raced);
     if (kMode == kWeightResidual) qw.load(qrow, q, V, base_v, raced);
     const uint4 r = philox(draw_counter(a.position, a.req, SPEC_PURPOSE_SAMPLE, (uint32_t)q), a.k0, a.k1);
@@ -546,11 +494,11 @@ __device__ void race_level1_impl(const void* row, const void* qrow, int q_dtype,
   }
 }
 
-template <typename T, typename Q, int kMode, int kSrc>
+template <typename T, typename Q, int kMode>
 __device__ __forceinline__ void race_level1(const void* row, const void* qrow, int q_dtype, int V, int base_v,
                                             int q_first, int q_end, int warp_id, int nwarps, const RaceArgs& a,
                                             KeyState& best) {
-  race_level1_impl<T, Q, kMode, kSrc, false, false>(row, qrow, q_dtype, V, base_v, q_first, q_end, warp_id, nwarps, a,
+  race_level1_impl<T, Q, kMode, false, false>(row, qrow, q_dtype, V, base_v, q_first, q_end, warp_id, nwarps, a,
                                                     best, best, 0, true);
 }
 
@@ -669,10 +617,10 @@ __device__ void race_level1_any(const VerifyLaunch& p, const void* row, const vo
                                 int warp_id, int nwarps, const RaceArgs& a, KeyState& best) {
   if (p.vec_s) {
     if (kMode == kWeightResidual && p.q_dtype == SPEC_F32)
-      race_level1<T, float, kMode, kSrcGlobalVec>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id, nwarps, a,
+      race_level1<T, float, kMode>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id, nwarps, a,
                                                   best);
     else
-      race_level1<T, __nv_bfloat16, kMode, kSrcGlobalVec>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id,
+      race_level1<T, __nv_bfloat16, kMode>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id,
                                                           nwarps, a, best);
   } else {
     race_level1_scalar<T, kMode, false, false>(row, qrow, p.q_dtype, p.V, 0, q_first, q_end, warp_id, nwarps, a, best,
