@@ -81,12 +81,13 @@ __device__ __forceinline__ double units_to_double(long long units) {
 // ---------------------------------------------------------------------------
 // Batches of more than 1024 draft positions or 1024 requests
 // ---------------------------------------------------------------------------
-// One thread-block cluster of C = ceil(max(B * K, B) / 1024) <= 8 CTAs, one
-// draft key per thread: CTA c owns the draft slots e = i * K + (k - 1) in
-// [1024 c, 1024 c + 1024) and the requests of that index range.  A single CTA
-// is bound by its serial searches (eight keys a thread) and by shared-memory
-// bank conflicts; eight CTAs take one key a thread and exchange through
-// distributed shared memory, which one GPC's SMs reach without a trip to L2.
+// One thread-block cluster of C = 2, 4 or 8 CTAs, the least with
+// max(B * K, B) <= 1024 C, one draft key per thread: CTA c owns the draft slots
+// e = i * K + (k - 1) in [1024 c, 1024 c + 1024) and the requests of that index
+// range.  A single CTA is bound by its serial searches (eight keys a thread) and
+// by shared-memory bank conflicts; eight CTAs take one key a thread and exchange
+// through distributed shared memory, which one GPC's SMs reach without a trip
+// to L2.
 //   1. scores and keys of the CTA's slots; a merge tree over the per-request
 //      runs (already descending) sorts them locally;
 //   2. every CTA copies the others' sorted keys and finds each of its keys'
@@ -148,6 +149,7 @@ struct ClusterSmem {
 template <int C>
 __global__ void __launch_bounds__(kAllocThreads, 1) allocate_cluster_kernel(const AllocLaunch p) {
   extern __shared__ __align__(16) unsigned char smem_raw[];
+  static_assert(C > 1, "one CTA's worth of keys is allocate_small_kernel's");
   ClusterSmem& sm = *reinterpret_cast<ClusterSmem*>(smem_raw);
   const int B = p.B, K = p.K, NK = B * K, CS = K | 1;
   const int tid = threadIdx.x, c = blockIdx.x;
@@ -234,36 +236,32 @@ __global__ void __launch_bounds__(kAllocThreads, 1) allocate_cluster_kernel(cons
     dst = t;
     x = lds_u64(src + 8u * (uint32_t)tid);
   }
-  if (C > 1) {
-    sm.all[c][tid] = x;
-    cluster_sync_all();
-    // ---- the other CTAs' sorted keys, then this key's rank among them ----
+  sm.all[c][tid] = x;
+  cluster_sync_all();
+  // ---- the other CTAs' sorted keys, then this key's rank among them ----
 #pragma unroll
-    for (int o = 1; o < C; ++o) {
-      const int cc = (c + o) & (C - 1);
-      sm.all[cc][tid] = ldc_u64(cluster_addr((uint32_t)__cvta_generic_to_shared(&sm.all[cc][tid]), cc));
-    }
-    __syncthreads();
+  for (int o = 1; o < C; ++o) {
+    const int cc = (c + o) & (C - 1);
+    sm.all[cc][tid] = ldc_u64(cluster_addr((uint32_t)__cvta_generic_to_shared(&sm.all[cc][tid]), cc));
   }
+  __syncthreads();
   int rank = tid;
-  if (C > 1) {
-    uint32_t base[C];
-    int cnt[C];
+  uint32_t base[C];
+  int cnt[C];
 #pragma unroll
-    for (int o = 1; o < C; ++o) {
-      base[o] = (uint32_t)__cvta_generic_to_shared(sm.all[(c + o) & (C - 1)]);
-      cnt[o] = 0;
-    }
+  for (int o = 1; o < C; ++o) {
+    base[o] = (uint32_t)__cvta_generic_to_shared(sm.all[(c + o) & (C - 1)]);
+    cnt[o] = 0;
+  }
 #pragma unroll
-    for (int step = kSlots >> 1; step > 0; step >>= 1)
+  for (int step = kSlots >> 1; step > 0; step >>= 1)
 #pragma unroll
-      for (int o = 1; o < C; ++o)
-        if (lds_u64(base[o] + 8u * (uint32_t)(cnt[o] + step - 1)) > x) cnt[o] += step;
+    for (int o = 1; o < C; ++o)
+      if (lds_u64(base[o] + 8u * (uint32_t)(cnt[o] + step - 1)) > x) cnt[o] += step;
 #pragma unroll
-    for (int o = 1; o < C; ++o) {
-      if (lds_u64(base[o] + 8u * (uint32_t)cnt[o]) > x) ++cnt[o];
-      rank += cnt[o];
-    }
+  for (int o = 1; o < C; ++o) {
+    if (lds_u64(base[o] + 8u * (uint32_t)cnt[o]) > x) ++cnt[o];
+    rank += cnt[o];
   }
   const int xi = 0xFFFF - (int)(x & 0xFFFFull);
   const int xk = 0xFFFF - (int)((x >> 16) & 0xFFFFull);
@@ -290,13 +288,9 @@ __global__ void __launch_bounds__(kAllocThreads, 1) allocate_cluster_kernel(cons
     const long long part = lo > 0 ? prefix[lo - 1] : 0;
     const uint32_t mine = (uint32_t)__cvta_generic_to_shared(&sm.contrib[c][tid]);
 #pragma unroll
-    for (int o = 0; o < C; ++o) {
-      if (C > 1) stc_u64(cluster_addr(mine, o), (unsigned long long)part);
-      else sm.contrib[c][tid] = part;
-    }
+    for (int o = 0; o < C; ++o) stc_u64(cluster_addr(mine, o), (unsigned long long)part);
   }
-  if (C > 1) cluster_sync_all();
-  else __syncthreads();
+  cluster_sync_all();
 
   // ---- Eq. (dcut-select): first maximiser of U / cost, in every CTA ----
   if (tid < 32) {
@@ -336,19 +330,15 @@ __global__ void __launch_bounds__(kAllocThreads, 1) allocate_cluster_kernel(cons
     bool next = false;
     if (sk < K) {  // slot e + 1, in the next CTA past this one's last slot
       if (tid + 1 < kSlots) next = sm.slot_rank[tid + 1] < TD;
-      else if (C > 1) next = ldc_s32(cluster_addr((uint32_t)__cvta_generic_to_shared(&sm.slot_rank[0]), c + 1)) < TD;
+      else next = ldc_s32(cluster_addr((uint32_t)__cvta_generic_to_shared(&sm.slot_rank[0]), c + 1)) < TD;
     }
     if (!next) {
       const uint32_t d = (uint32_t)__cvta_generic_to_shared(&sm.depth[si]);
 #pragma unroll
-      for (int o = 0; o < C; ++o) {
-        if (C > 1) stc_s32(cluster_addr(d, o), sk);
-        else sm.depth[si] = sk;
-      }
+      for (int o = 0; o < C; ++o) stc_s32(cluster_addr(d, o), sk);
     }
   }
-  if (C > 1) cluster_sync_all();
-  else __syncthreads();
+  cluster_sync_all();
 
   // ---- row offsets: exclusive scan of (n_i + 1) over all requests, in every
   // CTA; each writes its requests' outputs ----
@@ -654,7 +644,9 @@ __global__ void __launch_bounds__(kAllocThreads) allocate_small_kernel(const All
 bool allocate_is_small(int B, int K) { return B <= kSmallSlots && (long long)B * K <= kSmallSlots; }
 
 // One cluster of C CTAs (B and B * K are at most 1024 C), launched behind the
-// previous kernel as launch_after_previous does.
+// previous kernel as launch_after_previous does.  The shared-memory limit is
+// raised on every call (it and the cluster attribute: at most 0.3 us of an 8.5 us
+// call): a note per device that it has been would be stale after a device reset.
 template <int C>
 static cudaError_t launch_cluster(const AllocLaunch& p, cudaStream_t stream) {
   cudaError_t err = cudaFuncSetAttribute(allocate_cluster_kernel<C>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -682,8 +674,7 @@ cudaError_t launch_allocate(const AllocLaunch& p, cudaStream_t stream) {
     err = launch_after_previous(allocate_small_kernel, dim3(1), dim3(kAllocThreads), 0, stream, p);
     return err != cudaSuccess ? err : cudaGetLastError();
   }
-  const int slots = std::max(p.B * p.K, p.B);
-  if (slots <= kSlots) return launch_cluster<1>(p, stream);
+  const int slots = std::max(p.B * p.K, p.B);  // > kSlots here
   if (slots <= 2 * kSlots) return launch_cluster<2>(p, stream);
   if (slots <= 4 * kSlots) return launch_cluster<4>(p, stream);
   return launch_cluster<8>(p, stream);
