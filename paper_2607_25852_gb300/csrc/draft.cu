@@ -604,7 +604,8 @@ extern "C" int spec_draft(const void* logits, int logits_dtype, int B, int K, in
   p.NC = g.NC;
   p.chunk = g.chunk;
   const size_t esize = logits_dtype == SPEC_F32 ? 4 : 2;
-  // 16-byte loads of each lane's 8 entries: aligned rows and whole 8-entry groups
+  // 16-byte loads: rows on the 16-byte grid, of whole groups of 8 entries.  (fp32
+  // rows of V % 8 == 4 lie on the grid too, but take the shifted words.)
   const bool vec = (reinterpret_cast<uintptr_t>(logits) & 15u) == 0 && ((size_t)V * esize) % 16 == 0 && V % 8 == 0;
   const cudaError_t err = logits_dtype == SPEC_F32 ? spec::launch_draft_typed<float>(p, vec, stream)
                                                    : spec::launch_draft_typed<__nv_bfloat16>(p, vec, stream);

@@ -141,7 +141,11 @@ static ShardGeometry shard_geometry(int B, int K, int Vs) {
   s.NC = (int)((Vs + chunk - 1) / chunk);  // every chunk non-empty
   s.chunk = (int)chunk;
   // at least a quad for each of a CTA's eight warps: a rank's round of 25136
-  // columns takes 31.5 us so, 32.1 us with three quads a CTA
+  // columns takes 31.5 us so, 32.1 us with three quads a CTA.  Off the 16-byte
+  // grid a warp step is one block, so eight quads are four steps a warp: shard 3
+  // of 8 of V = 201087 still gains (31.0 / 32.5 us), others lose (shard 6 of 8 of
+  // V = 65537, B = 96, K = 4 28.8 / 24.8; shard 2 of 4 of V = 128257, fp32, B = 32,
+  // K = 8 28.8 / 27.3).
   s.quads_s = std::max(kSampleThreads / 32, g.chunk_s / kRaceQuad);
   // a shard of Vs columns spans at most ceil(Vs / 1024) + 1 quads
   const long long nq_max = (Vs + kRaceQuad - 1) / kRaceQuad + 1;

@@ -96,7 +96,8 @@ VerifyGeometry verify_geometry(int B, int K, int V) {
   long long chunk_s = round_up(ceil_div(V, ncs), 1024);
   // A CTA's eight warps take a quad each at a time: whole rounds of eight
   // quads, if the CTAs still fit one wave of four per SM (B=32, V=151936, dense
-  // q: 28.5 us a call with eight quads a CTA, 29.5 with nine).
+  // q: 28.5 us a call with eight quads a CTA, 29.5 with nine; V=151935, off the
+  // 16-byte grid, where a warp step is a block: 26.5 / 27.7).
   const long long even = chunk_s / 8192 * 8192;
   if (even > 0 && ceil_div(V, even) * B <= 608) chunk_s = even;
   ncs = ceil_div(V, chunk_s);
